@@ -459,8 +459,8 @@ tc_status tc_sample_estimate_q(const tc_graph* g, const tc_motif* motif, int64_t
  *
  * Graphs are borrowed: they must outlive the batch.  The batch owns device
  * memory for each distinct weights key (prefix and index, 8 (m + 1) plus
- * tc_sample_index_bytes) and 4 k bytes of sample order per query with
- * k >= 65536; k may be at most 2^40.
+ * tc_sample_index_bytes) and about 4.6 k bytes of sample order per query
+ * with k >= 65536; k may be at most 2^40.
  */
 typedef struct {
   const tc_graph* graph;

@@ -32,7 +32,14 @@ struct Query {
   tc_query q;
   Plan plan;
   int slot;
-  uint32_t* order;  // key order (chunk after chunk) or NULL
+};
+
+// A work record of the sampling launch: a query's samples in id order, or
+// one chunk of them in key order.
+struct Record {
+  int query;
+  uint64_t base, count;  // samples [base, base + count) of the query
+  void* order;           // order_bytes(count) bytes, or NULL (id order)
 };
 
 constexpr int kBlockSizes[3] = {128, 256, 512};
@@ -43,21 +50,26 @@ constexpr uint32_t kTiles[3] = {2048, 8192, 32768};
 struct tc_batch {
   std::vector<Query> queries;
   std::vector<Slot> slots;
+  std::vector<Record> work;
+  std::vector<char> h_records;     // kBatchQueryBytes each, as in device memory
   std::vector<void*> allocations;  // every cudaMalloc of the batch
   uint64_t device_bytes = 0;
   void* scan_scratch = nullptr;    // tile states of the weights scan, for the largest graph
   void* sort_scratch = nullptr;
   uint32_t* err = nullptr;         // one error word per slot
-  char* records = nullptr;         // nq * kBatchQueryBytes
-  uint64_t* tile_begin = nullptr;  // nq + 1
-  unsigned long long* next_item = nullptr;
+  char* records = nullptr;         // work.size() * kBatchQueryBytes
+  // the records of graphs with 64-bit list times [0, n64), then those with
+  // 32-bit times: a launch each, with its own item numbering and counter
+  uint32_t n64 = 0;
+  uint64_t* tile_begin = nullptr;  // work.size() + 2: each kind's numbering ends with its total
+  unsigned long long* next_item = nullptr;  // 2
   SampleSums* sums = nullptr;      // nq
   SampleSums* h_sums = nullptr;    // pinned, nq
   uint64_t* h_W = nullptr;         // pinned, one per slot
   uint32_t* h_err = nullptr;       // pinned, one per slot
   int block_size = 256;
   uint32_t tile = 8192;
-  unsigned blocks = 0;
+  unsigned blocks[2] = {0, 0};
   bool use_graph = true;
   cudaStream_t cap = nullptr;
   cudaGraph_t graph = nullptr;
@@ -97,14 +109,17 @@ void batch_free(tc_batch* b) {
 
 // Item numbering for the current tile size.
 tc_status upload_tiles(tc_batch* b) {
-  std::vector<uint64_t> tb(b->queries.size() + 1, 0);
-  for (size_t q = 0; q < b->queries.size(); q++) tb[q + 1] = tb[q] + (b->queries[q].q.k + b->tile - 1) / b->tile;
+  const uint32_t split[3] = {0, b->n64, (uint32_t)b->work.size()};
+  std::vector<uint64_t> tb;
+  for (int kind = 0; kind < 2; kind++) {
+    tb.push_back(0);
+    for (uint32_t r = split[kind]; r < split[kind + 1]; r++)
+      tb.push_back(tb.back() + batch_record_items(b->h_records.data() + kBatchQueryBytes * r, b->tile));
+    const int bps = sample_batch_blocks_per_sm(b->block_size, kind == 1);
+    if (bps == 0) return set_error(TC_ERR_INVALID_ARG, "batch block size must be 128, 256 or 512");
+    b->blocks[kind] = (unsigned)std::min<uint64_t>((uint64_t)num_sms() * bps, std::max<uint64_t>(tb.back(), 1));
+  }
   TC_CUDA(cudaMemcpy(b->tile_begin, tb.data(), sizeof(uint64_t) * tb.size(), cudaMemcpyHostToDevice));
-  const int bps = sample_batch_blocks_per_sm(b->block_size);
-  if (bps == 0) return set_error(TC_ERR_INVALID_ARG, "batch block size must be 128, 256 or 512");
-  uint64_t blocks = (uint64_t)num_sms() * bps;
-  const uint64_t need = (tb.back() ? tb.back() : 1);
-  b->blocks = (unsigned)std::min<uint64_t>(blocks, need);
   return TC_OK;
 }
 
@@ -116,27 +131,29 @@ tc_status enqueue_prologue(tc_batch* b, cudaStream_t st) {
   TC_CUDA(cudaMemsetAsync(b->err, 0, sizeof(uint32_t) * ns, st));
   for (size_t s = 0; s < ns; s++) {
     const Slot& S = b->slots[s];
-    const uint64_t m = (uint64_t)S.g->m;
     EdgeWin* win = (EdgeWin*)(S.index + kIndexHeaderBytes);
     TC_TRY(launch_weights_scan(S.g, S.plan, S.delta, win, S.prefix, nullptr, b->scan_scratch, b->err + s, st));
     TC_TRY(launch_guide(S.g, S.plan, S.delta, S.prefix, S.index, b->err + s, st));
   }
-  for (const Query& Q : b->queries) {
-    if (!Q.order) continue;
-    const Slot& S = b->slots[Q.slot];
-    for (uint64_t base = 0; base < Q.q.k; base += kChunkSamples) {
-      const uint64_t count = std::min<uint64_t>(Q.q.k - base, kChunkSamples);
-      TC_TRY(sort_sample_ids((const IndexHeader*)S.index, Q.q.seed, Q.q.sample_offset + base, count, b->sort_scratch,
-                             Q.order + base, st));
-    }
+  for (const Record& R : b->work) {
+    if (!R.order) continue;
+    const tc_query& q = b->queries[R.query].q;
+    TC_TRY(order_samples(q.seed, q.sample_offset + R.base, R.count, 1, b->sort_scratch, R.order, st));
   }
   return TC_OK;
 }
 
 tc_status enqueue_sampling(tc_batch* b, cudaStream_t st) {
-  TC_CUDA(cudaMemsetAsync(b->next_item, 0, sizeof(unsigned long long), st));
-  return launch_sample_batch(b->block_size, b->tile, b->blocks, b->records, b->tile_begin,
-                             (uint32_t)b->queries.size(), b->next_item, b->sums, st);
+  // the persistent launch counts the work items itself: the buckets' own counters stay unused
+  TC_CUDA(cudaMemsetAsync(b->next_item, 0, 2 * sizeof(unsigned long long), st));
+  const uint32_t n = (uint32_t)b->work.size();
+  if (b->n64)
+    TC_TRY(launch_sample_batch(b->block_size, false, b->tile, b->blocks[0], b->records, b->tile_begin, b->n64,
+                               b->next_item, st));
+  if (n > b->n64)
+    TC_TRY(launch_sample_batch(b->block_size, true, b->tile, b->blocks[1], b->records + kBatchQueryBytes * b->n64,
+                               b->tile_begin + b->n64 + 1, n - b->n64, b->next_item + 1, st));
+  return TC_OK;
 }
 
 tc_status enqueue_epilogue(tc_batch* b, cudaStream_t st) {
@@ -232,11 +249,10 @@ tc_status capture(tc_batch* b) {
 tc_status create(const tc_query* hq, int64_t nq, const tc_batch_options* opts, cudaStream_t st, tc_batch* b) {
   // queries and their weight slots
   std::map<std::tuple<uint64_t, int, int, int, int, int, int64_t>, int> slot_of;
-  uint64_t max_m = 0, max_sort = 0, order_words = 0;
+  uint64_t max_m = 0, sort_bytes = 0, all_orders = 0;
   for (int64_t i = 0; i < nq; i++) {
     Query Q;
     Q.q = hq[i];
-    Q.order = nullptr;
     if (!Q.q.graph) return set_error(TC_ERR_INVALID_ARG, "query graph is NULL");
     TC_TRY(compile_plan_checked(&Q.q.motif, &Q.plan));
     if (Q.q.delta < 0) return set_error(TC_ERR_INVALID_ARG, "delta must be >= 0");
@@ -256,9 +272,14 @@ tc_status create(const tc_query* hq, int64_t nq, const tc_batch_options* opts, c
       max_m = std::max<uint64_t>(max_m, (uint64_t)S.g->m);
     }
     Q.slot = it->second;
-    if (Q.q.k >= kSortedMinSamples) {
-      max_sort = std::max<uint64_t>(max_sort, std::min<uint64_t>(Q.q.k, kChunkSamples));
-      order_words += (Q.q.k + 63) & ~63ull;  // 256-byte aligned starts
+    const uint64_t chunk = Q.q.k >= kBatchOrderedMinSamples ? kChunkSamples : Q.q.k;
+    for (uint64_t base = 0; base < Q.q.k; base += chunk) {
+      Record R{(int)i, base, std::min<uint64_t>(Q.q.k - base, chunk), nullptr};
+      if (Q.q.k >= kBatchOrderedMinSamples) {
+        sort_bytes = std::max<uint64_t>(sort_bytes, order_scratch_bytes(R.count, 1));
+        all_orders += order_bytes(R.count, 1);  // multiples of 256 bytes
+      }
+      b->work.push_back(R);
     }
     b->queries.push_back(Q);
   }
@@ -270,37 +291,40 @@ tc_status create(const tc_query* hq, int64_t nq, const tc_batch_options* opts, c
   }
   TC_TRY(batch_alloc(b, (void**)&b->scan_scratch, weights_scan_scratch_bytes(max_m)));
   TC_TRY(batch_alloc(b, (void**)&b->err, sizeof(uint32_t) * b->slots.size()));
-  if (max_sort) TC_TRY(batch_alloc(b, &b->sort_scratch, sort_scratch_bytes(max_sort)));
-  uint32_t* order = nullptr;
-  if (order_words) TC_TRY(batch_alloc(b, (void**)&order, sizeof(uint32_t) * order_words));
-  for (Query& Q : b->queries) {
-    if (Q.q.k < kSortedMinSamples) continue;
-    Q.order = order;
-    order += (Q.q.k + 63) & ~63ull;
+  if (sort_bytes) TC_TRY(batch_alloc(b, &b->sort_scratch, sort_bytes));
+  char* order = nullptr;
+  if (all_orders) TC_TRY(batch_alloc(b, (void**)&order, all_orders));
+  for (Record& R : b->work) {
+    if (b->queries[R.query].q.k < kBatchOrderedMinSamples) continue;
+    R.order = order;
+    order += order_bytes(R.count, 1);
   }
-  TC_TRY(batch_alloc(b, (void**)&b->records, kBatchQueryBytes * (size_t)nq));
-  TC_TRY(batch_alloc(b, (void**)&b->tile_begin, sizeof(uint64_t) * (size_t)(nq + 1)));
-  TC_TRY(batch_alloc(b, (void**)&b->next_item, sizeof(unsigned long long)));
+  TC_TRY(batch_alloc(b, (void**)&b->records, kBatchQueryBytes * b->work.size()));
+  TC_TRY(batch_alloc(b, (void**)&b->tile_begin, sizeof(uint64_t) * (b->work.size() + 2)));
+  TC_TRY(batch_alloc(b, (void**)&b->next_item, 2 * sizeof(unsigned long long)));
   TC_TRY(batch_alloc(b, (void**)&b->sums, sizeof(SampleSums) * (size_t)nq));
   TC_CUDA(cudaMallocHost((void**)&b->h_sums, sizeof(SampleSums) * (size_t)(nq ? nq : 1)));
   TC_CUDA(cudaMallocHost((void**)&b->h_W, sizeof(uint64_t) * (b->slots.size() + 1)));
   TC_CUDA(cudaMallocHost((void**)&b->h_err, sizeof(uint32_t) * (b->slots.size() + 1)));
-  {  // per-query argument records
-    std::vector<char> rec(kBatchQueryBytes * (size_t)nq);
-    for (int64_t i = 0; i < nq; i++) {
-      const Query& Q = b->queries[i];
-      const Slot& S = b->slots[Q.slot];
-      batch_query_record(rec.data() + kBatchQueryBytes * i, Q.q.graph, Q.plan, Q.q.delta, S.prefix, S.index, Q.q.k,
-                         Q.q.seed, Q.q.sample_offset, Q.order);
-    }
-    TC_CUDA(cudaMemcpy(b->records, rec.data(), rec.size(), cudaMemcpyHostToDevice));
+  // the work records, those with 64-bit list times first
+  b->n64 = (uint32_t)(std::stable_partition(b->work.begin(), b->work.end(),
+                                            [&](const Record& R) { return !b->queries[R.query].q.graph->pair_t32; }) -
+                      b->work.begin());
+  b->h_records.resize(kBatchQueryBytes * b->work.size());
+  for (size_t r = 0; r < b->work.size(); r++) {
+    const Record& R = b->work[r];
+    const Query& Q = b->queries[R.query];
+    const Slot& S = b->slots[Q.slot];
+    batch_query_record(b->h_records.data() + kBatchQueryBytes * r, Q.q.graph, Q.plan, Q.q.delta, S.prefix, S.index,
+                       Q.q.seed, Q.q.sample_offset, R.base, R.count, R.order, b->sums + R.query);
   }
+  TC_CUDA(cudaMemcpy(b->records, b->h_records.data(), b->h_records.size(), cudaMemcpyHostToDevice));
   for (cudaEvent_t& e : b->ev) TC_CUDA(cudaEventCreate(&e));
   // launch shape
   const int bs = opts ? opts->block_size : 0;
   const uint32_t tile = opts ? opts->tile : 0;
   b->use_graph = opts ? opts->use_graph != 0 : true;
-  if (bs && !sample_batch_blocks_per_sm(bs)) return set_error(TC_ERR_INVALID_ARG, "block_size must be 128, 256 or 512");
+  if (bs && !sample_batch_blocks_per_sm(bs, true)) return set_error(TC_ERR_INVALID_ARG, "block_size must be 128, 256 or 512");
   if (tile && (tile % (bs ? bs : 512)) != 0) return set_error(TC_ERR_INVALID_ARG, "tile must be a multiple of block_size");
   b->block_size = bs ? bs : 256;
   b->tile = tile ? tile : 8192;

@@ -402,28 +402,51 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
                          SampleSums* d_sums, cudaStream_t st, const void* qindex = nullptr,
                          const uint16_t* h = nullptr, unsigned long long* bins = nullptr);
 
-// Key-ordered sampling: samples are processed in chunks of at most
-// kChunkSamples, each put in key order by sort_sample_ids (no allocation;
-// scratch of sort_scratch_bytes(count)); calls below kSortedMinSamples
-// samples run in id order.
-constexpr uint64_t kSortedMinSamples = 1ull << 16;
+// Ordered sampling: samples are processed in chunks of at most kChunkSamples,
+// each partitioned by order_samples into nb = nb1 nb2 buckets of neighbouring
+// middle-edge draws (no allocation: an order of order_bytes, scratch of
+// order_scratch_bytes bytes for the same count and wave; few buckets come as
+// a multiple of wave).  Calls below kOrderedMinSamples samples run in id
+// order (nb = 0): the order costs two launches and the sampler's tiles a few
+// microseconds each, which neighbouring samples only win back beyond about
+// 5e5 samples (4e5 samples of a 1e7-edge graph: 65 us in id order, 71 + 15 us
+// ordered; 1e6: 147 us against 100 + 16 us).  In a batch, where the order
+// passes of all queries run back to back and the sampler's blocks always find
+// work, queries of 65,536 samples on are ordered.  sizes[b] ids of bucket b
+// start at ids[b room]; head[0] is set when a bucket outgrew its room (the
+// order is then not used), head[1] counts the buckets taken.
+struct OrderView {
+  uint32_t* head;
+  const uint32_t* sizes;
+  const uint32_t* ids;
+  uint32_t nb, nb1, nb2, room;
+};
+constexpr uint64_t kOrderedMinSamples = 1ull << 19;
+constexpr uint64_t kBatchOrderedMinSamples = 1ull << 16;
 constexpr uint64_t kChunkSamples = 1ull << 28;
-size_t sort_scratch_bytes(uint64_t count);
-tc_status sort_sample_ids(const IndexHeader* hdr, uint64_t seed, uint64_t first, uint64_t count, void* scratch,
-                          uint32_t* order, cudaStream_t st);
+size_t order_bytes(uint64_t count, uint32_t wave);
+size_t order_scratch_bytes(uint64_t count, uint32_t wave);
+OrderView order_view(uint64_t count, uint32_t wave, void* order);
+tc_status order_samples(uint64_t seed, uint64_t first, uint64_t count, uint32_t wave, void* scratch, void* order,
+                        cudaStream_t st);
 
-// Batched sampling: each query's arguments are a kBatchQueryBytes-byte
-// record in device memory, written on the host by batch_query_record; the
-// queries' work items (tiles of `tile` samples) are numbered query after
-// query, query q owning items [tile_begin[q], tile_begin[q + 1]).  order is
-// the query's key order (chunk after chunk) or NULL for id order.
+// Batched sampling: each record is the arguments of one query's samples
+// [chunk_base, chunk_base + count) (one chunk of them, in key order, or all
+// of them in id order), kBatchQueryBytes bytes in device memory, written on
+// the host by batch_query_record; its sums are added to *sums.  The records'
+// work items (groups of buckets holding about `tile` samples, or tiles of
+// `tile` ids) are numbered record after record, record q owning items
+// [tile_begin[q], tile_begin[q + 1]).
 constexpr size_t kBatchQueryBytes = 512;
 void batch_query_record(void* h_rec, const tc_graph* g, const Plan& plan, int64_t delta, const uint64_t* prefix,
-                        const void* index, uint64_t k, uint64_t seed, uint64_t offset, const uint32_t* order);
-int sample_batch_blocks_per_sm(int block_size);  // 0: unsupported block size
-tc_status launch_sample_batch(int block_size, uint32_t tile, unsigned blocks, const void* d_records,
+                        const void* index, uint64_t seed, uint64_t offset, uint64_t chunk_base, uint64_t count,
+                        void* order, SampleSums* sums);
+uint64_t batch_record_items(const void* h_rec, uint32_t tile);
+// One launch takes records of one kind (compact or not).
+int sample_batch_blocks_per_sm(int block_size, bool compact);  // 0: unsupported block size
+tc_status launch_sample_batch(int block_size, bool compact, uint32_t tile, unsigned blocks, const void* d_records,
                               const uint64_t* d_tile_begin, uint32_t nq, unsigned long long* d_next_item,
-                              SampleSums* d_sums, cudaStream_t st);
+                              cudaStream_t st);
 
 // Diagnostic timing by phase (tc_set_timing, tc_last_phase_ms): a
 // PhaseTimer records an event pair around each start()/stop() on its stream

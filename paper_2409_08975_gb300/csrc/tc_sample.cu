@@ -2,6 +2,8 @@
 // sampler with CheckMotif / ListCount and the reduction of X (Alg. 2-5).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <utility>
 #include <vector>
@@ -496,9 +498,9 @@ struct SamplerArgs {
   const EdgeWin* win;
   const uint32_t* guide;
   uint64_t k, seed, offset;
-  const uint32_t* order;  // processing order of the chunk's samples (NULL: in id order)
   uint64_t chunk_base;    // index of the chunk's first sample within the call
   uint64_t count;         // samples in the chunk
+  OrderView ord;          // the chunk's samples by buckets of their draws (nb = 0: in id order)
   uint32_t m;
   int64_t delta;
   uint64_t graph_id;
@@ -513,57 +515,72 @@ struct SamplerArgs {
   const IndexHeader* rec_hdr;
 };
 
-// Two bisections of [s, e) at once: *a = the first position with time > xa,
-// *b = the first with time > xb (incl) or >= xb; one probe of each per step.
-template <class TimeAt>
-__device__ __forceinline__ void search_time2(uint32_t s, uint32_t e, int64_t xa, int64_t xb, bool incl, TimeAt tt,
-                                             uint32_t* a, uint32_t* b) {
-  uint32_t la = s, ha = e, lb = s, hb = e;
-  while (la < ha || lb < hb) {
-    const uint32_t ma = la + ((ha - la) >> 1), mb = lb + ((hb - lb) >> 1);
-    const bool ra = la < ha, rb = lb < hb;
-    const int64_t va = ra ? tt(ma) : 0, vb = rb ? tt(mb) : 0;
-    if (ra) {
-      if (va <= xa) la = ma + 1; else ha = ma;
-    }
-    if (rb) {
-      if (incl ? vb <= xb : vb < xb) lb = mb + 1; else hb = mb;
-    }
+// Times inside the sampler: t - tmin in 32 bits on graphs with 32-bit list
+// times (Compact; every time, sum and comparison is then one 32-bit
+// operation), else the int64 times.
+template <bool Compact>
+struct SampleTime {
+  typedef uint32_t T;
+  static __device__ __forceinline__ T rel(const SamplerArgs& A, int64_t t) { return (uint32_t)t - (uint32_t)A.tmin; }
+  static __device__ __forceinline__ T pair(const SamplerArgs& A, uint32_t p) { return __ldg(A.pair_t32 + p); }
+  static __device__ __forceinline__ bool beyond(const SamplerArgs& A, T first, T last) {
+    return (uint64_t)(last - first) > (uint64_t)A.delta;  // first <= last
   }
-  *a = la;
-  *b = lb;
-}
+  // first + delta; every list time is at most 2^32 - 1
+  static __device__ __forceinline__ T end(const SamplerArgs& A, T first) {
+    const uint64_t x = (uint64_t)first + (uint64_t)A.delta;  // delta < 2^63
+    return x > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)x;
+  }
+  static __device__ __forceinline__ int64_t absolute(const SamplerArgs& A, T t) { return (int64_t)t + A.tmin; }
+};
+template <>
+struct SampleTime<false> {
+  typedef int64_t T;
+  static __device__ __forceinline__ T rel(const SamplerArgs&, int64_t t) { return t; }
+  static __device__ __forceinline__ T pair(const SamplerArgs& A, uint32_t p) { return __ldg(A.pair_t + p); }
+  static __device__ __forceinline__ bool beyond(const SamplerArgs& A, T first, T last) {
+    return (uint64_t)last - (uint64_t)first > (uint64_t)A.delta;
+  }
+  static __device__ __forceinline__ T end(const SamplerArgs& A, T first) { return sat_add(first, A.delta); }
+  static __device__ __forceinline__ int64_t absolute(const SamplerArgs&, T t) { return t; }
+};
 
-// Positions [a, b) of the pair list L_{x,y} with time in (tlo, thi) or
-// (tlo, thi] (hi_incl).  The list's range comes from the pair hash table (one
-// 16-byte slot per probe).  Returns false when x never sends to y.
-__device__ __forceinline__ bool pair_window(const SamplerArgs& A, int32_t x, int32_t y, int64_t tlo, int64_t thi,
-                                            bool hi_incl, uint32_t* a, uint32_t* b) {
-  const uint64_t key = pair_key((uint32_t)x, (uint32_t)y);
-  uint64_t h = mix64(key) & A.hash_mask;
-  uint32_t s = 0, e = 0;
-  bool found = false;
+// Positions [*s, *e) of the pair list L_{x,y} (empty when x never sends to
+// y) from the pair hash table, one 16-byte slot per probe.
+__device__ __forceinline__ void pair_list(const SamplerArgs& A, int32_t x, int32_t y, uint32_t* s, uint32_t* e) {
+  *s = *e = 0;
+  uint64_t h = mix64(pair_key((uint32_t)x, (uint32_t)y)) & A.hash_mask;
   for (uint64_t probe = 0; probe <= A.hash_mask; probe++) {
     const uint4 slot = __ldg(reinterpret_cast<const uint4*>(A.pair_hash + h));
     if (slot.x == (uint32_t)x && slot.y == (uint32_t)y) {
-      s = slot.z;
-      e = slot.w;
-      found = true;
-      break;
+      *s = slot.z;
+      *e = slot.w;
+      return;
     }
-    if (slot.x == 0xFFFFFFFFu) break;
+    if (slot.x == 0xFFFFFFFFu) return;
     h = (h + 1) & A.hash_mask;
   }
-  if (!found) return false;
-  // both bounds bisect [s, e) in lockstep, so that their probes are in flight together
-  if (A.pair_t32) {  // 4-byte entries, eight per sector
-    auto tt = [&](uint32_t p) { return (int64_t)__ldg(A.pair_t32 + p) + A.tmin; };
-    search_time2(s, e, tlo, thi, hi_incl, tt, a, b);
-  } else {
-    auto tt = [&](uint32_t p) { return __ldg(A.pair_t + p); };
-    search_time2(s, e, tlo, thi, hi_incl, tt, a, b);
+}
+
+// Positions [*a, *b) of the non-empty pair list [s, e) with time in (tlo,
+// thi]: the first positions with time > tlo and with time > thi.  Both
+// bisections halve the same length, so one loop runs them with a probe of
+// each in flight.
+template <bool Compact>
+__device__ __forceinline__ void pair_window(const SamplerArgs& A, uint32_t s, uint32_t e,
+                                            typename SampleTime<Compact>::T tlo, typename SampleTime<Compact>::T thi,
+                                            uint32_t* a, uint32_t* b) {
+  typedef SampleTime<Compact> Tm;
+  uint32_t pa = s, pb = s;
+  for (uint32_t len = e - s; len > 1;) {
+    const uint32_t half = len >> 1;
+    const typename Tm::T va = Tm::pair(A, pa + half - 1), vb = Tm::pair(A, pb + half - 1);
+    if (va <= tlo) pa += half;
+    if (vb <= thi) pb += half;
+    len -= half;
   }
-  return true;
+  *a = pa + (Tm::pair(A, pa) <= tlo ? 1u : 0u);
+  *b = pb + (Tm::pair(A, pb) <= thi ? 1u : 0u);
 }
 
 // ListCount (Alg. 4) over l lists by one merged pass in time order: an
@@ -601,44 +618,75 @@ __device__ uint64_t list_count_merge(const int64_t* __restrict__ pt, const uint3
   return acc[l];
 }
 
-// ListCount of a gap with two or more lists (kept out of line so that its
-// arrays do not weigh on the single-list path).
+// The same over two lists: for every element of the second, the elements of
+// the first that are strictly earlier (a forward pointer; at most 2^64 - 1
+// pairs, as both lists have fewer than 2^32 entries).
+template <bool Compact>
+__device__ __forceinline__ uint64_t list_count_two(const SamplerArgs& A, uint32_t a0, uint32_t b0, uint32_t a1,
+                                                   uint32_t b1) {
+  typedef SampleTime<Compact> Tm;
+  uint64_t c = 0;
+  uint32_t p = a0;
+  typename Tm::T tp = Tm::pair(A, p);
+  for (uint32_t q = a1; q < b1; q++) {
+    const typename Tm::T tq = Tm::pair(A, q);
+    while (p < b0 && tp < tq) {
+      p++;
+      if (p < b0) tp = Tm::pair(A, p);
+    }
+    c += p - a0;
+  }
+  return c;
+}
+
+// ListCount of a gap with two or more lists, over times in (tlo, thi] (kept
+// out of line so that its arrays do not weigh on the single-list path).
+template <bool Compact>
 __device__ __noinline__ uint64_t gap_count_multi(const SamplerArgs& A, const Plan& P, int gp, int32_t up, int32_t u,
-                                                int32_t v, int32_t vp, int64_t tlo, int64_t thi, bool incl,
-                                                uint32_t* err) {
+                                                int32_t v, int32_t vp, typename SampleTime<Compact>::T tlo,
+                                                typename SampleTime<Compact>::T thi, uint32_t* err) {
   auto phi = [&](int role) { return role == 0 ? up : (role == 1 ? u : (role == 2 ? v : vp)); };
   const int l = P.ngap[gp];
   uint32_t a[16], b[16];
   for (int j = 0; j < l; j++) {
-    if (!pair_window(A, phi(P.gx[gp][j]), phi(P.gy[gp][j]), tlo, thi, incl, &a[j], &b[j])) return 0;
+    uint32_t s, e;
+    pair_list(A, phi(P.gx[gp][j]), phi(P.gy[gp][j]), &s, &e);
+    if (s == e) return 0;
+    pair_window<Compact>(A, s, e, tlo, thi, &a[j], &b[j]);
     if (a[j] == b[j]) return 0;
   }
+  if (l == 2) return list_count_two<Compact>(A, a[0], b[0], a[1], b[1]);
   return list_count_merge(A.pair_t, a, b, l, err);
 }
 
 // Product over the gaps of their ListCounts (Alg. 3, 4): gap gp holds the
 // non-anchor motif edges of ranks between anchor ranks NG gp and gp + 1, with
 // times in (ta[gp], ta[gp + 1]); the last gap runs up to ta[0] + delta
-// inclusive.  phi maps path roles (u', u, v, v') to graph vertices.
-template <int NG>
-__device__ __forceinline__ uint64_t gaps_product(const SamplerArgs& A, const Plan& P, const int64_t* ta, int32_t up,
-                                                 int32_t u, int32_t v, int32_t vp, uint32_t* err) {
+// inclusive.  The anchor times increase strictly, so an open upper bound t
+// is the closed bound t - 1.  phi maps path roles (u', u, v, v') to graph
+// vertices.
+template <int NG, bool Compact>
+__device__ __forceinline__ uint64_t gaps_product(const SamplerArgs& A, const Plan& P,
+                                                 const typename SampleTime<Compact>::T* ta, int32_t up, int32_t u,
+                                                 int32_t v, int32_t vp, uint32_t* err) {
+  typedef SampleTime<Compact> Tm;
   auto phi = [&](int role) { return role == 0 ? up : (role == 1 ? u : (role == 2 ? v : vp)); };
   uint64_t X = 1;
 #pragma unroll
   for (int gp = 0; gp < NG; gp++) {
     const int l = P.ngap[gp];
     if (l == 0) continue;
-    const int64_t tlo = ta[gp];
-    const int64_t thi = gp < NG - 1 ? ta[gp + 1] : sat_add(ta[0], A.delta);
-    const bool incl = gp == NG - 1;
+    const typename Tm::T tlo = ta[gp];
+    const typename Tm::T thi = gp < NG - 1 ? ta[gp + 1] - 1 : Tm::end(A, ta[0]);
     uint64_t c;
     if (l == 1) {  // one list: its length in the window
-      uint32_t a0, b0;
-      if (!pair_window(A, phi(P.gx[gp][0]), phi(P.gy[gp][0]), tlo, thi, incl, &a0, &b0)) return 0;
+      uint32_t s, e, a0, b0;
+      pair_list(A, phi(P.gx[gp][0]), phi(P.gy[gp][0]), &s, &e);
+      if (s == e) return 0;
+      pair_window<Compact>(A, s, e, tlo, thi, &a0, &b0);
       c = b0 - a0;
     } else {
-      c = gap_count_multi(A, P, gp, up, u, v, vp, tlo, thi, incl, err);
+      c = gap_count_multi<Compact>(A, P, gp, up, u, v, vp, tlo, thi, err);
     }
     if (c == 0) return 0;
     const uint64_t hi = __umul64hi(X, c);
@@ -650,60 +698,77 @@ __device__ __forceinline__ uint64_t gaps_product(const SamplerArgs& A, const Pla
 
 // CheckMotif of a wedge (3-vertex motif): base (u, v, t0) and second edge
 // to or from y at time tj; the three vertices distinct, t0 < tj <= t0 + delta.
+template <bool Compact>
 __device__ __forceinline__ uint64_t check_wedge(const SamplerArgs& A, const Plan& P, int32_t y, int32_t u, int32_t v,
-                                                int64_t t0, int64_t tj, uint32_t* err, uint32_t* checked) {
+                                                typename SampleTime<Compact>::T t0,
+                                                typename SampleTime<Compact>::T tj, uint32_t* err, uint32_t* checked) {
   if (u == v || y == u || y == v) return 0;
-  if (!(t0 < tj) || (uint64_t)tj - (uint64_t)t0 > (uint64_t)A.delta) return 0;
+  if (!(t0 < tj) || SampleTime<Compact>::beyond(A, t0, tj)) return 0;
   ++*checked;
-  const int64_t ta[2] = {t0, tj};
-  return gaps_product<2>(A, P, ta, y, u, v, y, err);
+  const typename SampleTime<Compact>::T ta[2] = {t0, tj};
+  return gaps_product<2, Compact>(A, P, ta, y, u, v, y, err);
 }
 
 // CheckMotif (Alg. 3) of the path (u' -e1- u -e2- v -e3- v'), or of the
 // wedge (u' -e1- u -e2- v) / (u -e2- v -e3- v') of a wedge anchor.
+template <bool Compact>
 __device__ __forceinline__ uint64_t check_motif(const SamplerArgs& A, const Plan& P, int32_t up, int32_t u,
-                                                int32_t v, int32_t vp, int64_t t1, int64_t t2, int64_t t3,
-                                                uint32_t* err, uint32_t* checked) {
+                                                int32_t v, int32_t vp, typename SampleTime<Compact>::T t1,
+                                                typename SampleTime<Compact>::T t2,
+                                                typename SampleTime<Compact>::T t3, uint32_t* err,
+                                                uint32_t* checked) {
   if (P.wedge)
-    return P.wedge == 1 ? check_wedge(A, P, up, u, v, t2, t1, err, checked)
-                        : check_wedge(A, P, vp, u, v, t2, t3, err, checked);
+    return P.wedge == 1 ? check_wedge<Compact>(A, P, up, u, v, t2, t1, err, checked)
+                        : check_wedge<Compact>(A, P, vp, u, v, t2, t3, err, checked);
   if (up == u || up == v || up == vp || u == v || u == vp || v == vp) return 0;
   // anchor edges ordered by rank must have strictly increasing times
-  int64_t ta[3];  // times of anchor ranks rk[0] < rk[1] < rk[2]
+  typename SampleTime<Compact>::T ta[3];  // times of anchor ranks rk[0] < rk[1] < rk[2]
 #pragma unroll
   for (int j = 0; j < 3; j++) {
     const int r = P.rk[j];
     ta[j] = r == P.e1 ? t1 : (r == P.mid ? t2 : t3);
   }
   if (!(ta[0] < ta[1] && ta[1] < ta[2])) return 0;
-  if ((uint64_t)ta[2] - (uint64_t)ta[0] > (uint64_t)A.delta) return 0;
+  if (SampleTime<Compact>::beyond(A, ta[0], ta[2])) return 0;
   ++*checked;
-  return gaps_product<3>(A, P, ta, up, u, v, vp, err);
+  return gaps_product<3, Compact>(A, P, ta, up, u, v, vp, err);
 }
 
 // The far vertex and time of the end edge at list position p of an alpha
 // list (alpha = 0: a wedge's dummy end, vertex -1).
-__device__ __forceinline__ void end_edge(const SamplerArgs& A, int alpha, uint32_t p, int32_t* x, int64_t* t) {
-  if (alpha < 0) {
-    const InEdge e = A.in_e[p];
-    *x = e.src;
-    *t = e.t;
-  } else if (alpha > 0) {
-    const OutEdge e = A.out_e[p];
-    *x = e.dst;
-    *t = e.t;
+template <bool Compact>
+__device__ __forceinline__ void end_edge(const SamplerArgs& A, int alpha, uint32_t p, int32_t* x,
+                                         typename SampleTime<Compact>::T* t) {
+  if (alpha != 0) {
+    const int4 e = __ldg(reinterpret_cast<const int4*>(alpha < 0 ? (const void*)(A.in_e + p) : (const void*)(A.out_e + p)));
+    *x = alpha < 0 ? e.x : e.y;
+    *t = SampleTime<Compact>::rel(A, (int64_t)(((uint64_t)(uint32_t)e.w << 32) | (uint32_t)e.z));
   } else {
     *x = -1;
     *t = 0;
   }
 }
 
-// Per-thread running sums of a sampling kernel.
+// Per-thread running sums of a sampling kernel; errors go to the block's word.
 struct ThreadSums {
-  uint64_t sx = 0, hits = 0;
-  uint32_t checked = 0;
+  uint64_t sx = 0;
   unsigned __int128 sx2 = 0;
-  uint32_t err = 0;
+  uint32_t hits = 0, checked = 0;  // a thread takes fewer than 2^32 samples
+  uint32_t* s_err;
+  __device__ __forceinline__ explicit ThreadSums(uint32_t* e) : s_err(e) {}
+  __device__ __forceinline__ void clear() {
+    sx = 0;
+    sx2 = 0;
+    hits = checked = 0;
+  }
+  __device__ __forceinline__ void fail(uint32_t bits) { atomicOr(s_err, bits); }
+  __device__ __forceinline__ void add(uint64_t X) {
+    if (X == 0) return;
+    sx += X;
+    if (sx < X) fail(kErrOverflow);
+    sx2 += (unsigned __int128)X * X;
+    hits++;
+  }
 };
 
 // The index must have been built for this graph, anchor class and delta
@@ -719,11 +784,10 @@ __device__ __forceinline__ uint32_t index_check(const SamplerArgs& A, const Plan
   return (matches(H) && (A.rec_hdr == nullptr || matches(A.rec_hdr))) ? 0u : kErrIndexMismatch;
 }
 
-// Resident blocks per SM the sampler is compiled for (caps its registers).
+// Resident blocks of 512 threads per SM the sampler is compiled for (caps its registers).
 #ifndef TC_SAMPLE_MIN_BLOCKS
-#define TC_SAMPLE_MIN_BLOCKS 4
+#define TC_SAMPLE_MIN_BLOCKS 3
 #endif
-#define TC_SAMPLE_MIN_BLOCKS_DECL TC_SAMPLE_MIN_BLOCKS
 
 // Warp-shuffle reduction of the per-thread sums, one shared atomic per warp
 // and one global atomic per block; 128-bit sum of squares with carries,
@@ -778,7 +842,8 @@ __device__ __forceinline__ void block_commit(SampleSums* G, uint64_t W, uint64_t
 // (p - prefix[e])-th pair (p1, p3) of middle edge e, p1 major; the sum of
 // CheckMotif over all paths is the exact count C, the sum of squares gives
 // the exact variance of one sample.  Paths [first, first + count).
-__global__ void __launch_bounds__(256, TC_SAMPLE_MIN_BLOCKS_DECL) k_path_sum(const __grid_constant__ SamplerArgs A,
+template <bool Compact>
+__global__ void __launch_bounds__(256, 4) k_path_sum(const __grid_constant__ SamplerArgs A,
                                                                             const __grid_constant__ Plan P,
                                                                             uint64_t first, uint64_t count) {
   const IndexHeader* H = A.hdr;
@@ -796,10 +861,7 @@ __global__ void __launch_bounds__(256, TC_SAMPLE_MIN_BLOCKS_DECL) k_path_sum(con
     if (threadIdx.x == 0) atomicOr(&A.sums->err, bad);
     return;
   }
-  uint64_t sx = 0, hits = 0;
-  uint32_t checked = 0;
-  unsigned __int128 sx2 = 0;
-  uint32_t err = 0;
+  ThreadSums T(&s_err);
   const uint64_t end = first + count < W ? first + count : W;
   for (uint64_t p = first + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < end;
        p += (uint64_t)gridDim.x * blockDim.x) {
@@ -809,36 +871,31 @@ __global__ void __launch_bounds__(256, TC_SAMPLE_MIN_BLOCKS_DECL) k_path_sum(con
       const uint32_t mid = lo + ((hi - lo + 1) >> 1);
       if (__ldg(A.prefix + mid) <= p) lo = mid; else hi = mid - 1;
     }
-    if (lo >= A.m) { err |= kErrBounds; continue; }
+    if (lo >= A.m) { T.fail(kErrBounds); continue; }
     const EdgeWin wn = A.win[lo];
     const OutEdge e = A.out_e[lo];
-    if (wn.d1 == 0 || wn.d3 == 0) { err |= kErrBounds; continue; }
+    if (wn.d1 == 0 || wn.d3 == 0) { T.fail(kErrBounds); continue; }
     const uint64_t j = p - __ldg(A.prefix + lo);
     const uint32_t p1 = wn.lo1 + (uint32_t)(j / wn.d3), p3 = wn.lo3 + (uint32_t)(j % wn.d3);
-    if (p1 >= A.m || p3 >= A.m) { err |= kErrBounds; continue; }
+    if (p1 >= A.m || p3 >= A.m) { T.fail(kErrBounds); continue; }
     int32_t up, vp;
-    int64_t t1, t3;
-    end_edge(A, P.alpha1, p1, &up, &t1);
-    end_edge(A, P.alpha3, p3, &vp, &t3);
-    const uint64_t X = check_motif(A, P, up, e.src, e.dst, vp, t1, e.t, t3, &s_err, &checked);
-    const uint64_t nx = sx + X;
-    if (nx < sx) err |= kErrOverflow;
-    sx = nx;
-    sx2 += (unsigned __int128)X * X;
-    hits += X != 0;
+    typename SampleTime<Compact>::T t1, t3;
+    end_edge<Compact>(A, P.alpha1, p1, &up, &t1);
+    end_edge<Compact>(A, P.alpha3, p3, &vp, &t3);
+    const uint64_t X = check_motif<Compact>(A, P, up, e.src, e.dst, vp, t1, SampleTime<Compact>::rel(A, e.t), t3,
+                                            &s_err, &T.checked);
+    T.add(X);
   }
-  block_commit(A.sums, W, sx, sx2, hits, checked, err, s_err, s_x, s_x2lo, s_x2hi, s_hits, s_checked);
+  block_commit(A.sums, W, T.sx, T.sx2, T.hits, T.checked, 0, s_err, s_x, s_x2lo, s_x2hi, s_hits, s_checked);
 }
 
 // The rejection loops: the first attempt is tested in the sampler itself and
 // these run only when it is rejected (probability below range / 2^64),
 // starting again from attempt 0.
-__device__ __forceinline__ bool bounded_draw_slow(uint64_t seed, uint64_t s, uint32_t draw, bool upper, uint64_t range,
-                                               uint64_t* out) {
-  return bounded_draw_words(seed, s, draw, upper, range, out);
+__device__ __noinline__ bool bounded_draw_slow(uint64_t seed, uint64_t s, uint64_t range, uint64_t* out) {
+  return bounded_draw_words(seed, s, 0, false, range, out);
 }
 
-// One sample (Alg. 2, 3): sample index i within the call (id offset + i).
 constexpr uint32_t kSmemBins = 1088;  // per-block bins of the proposal sampler (see k_sample): the 1,025 h of S = 1024
 constexpr size_t kSmemBinBytes = 3 * sizeof(unsigned long long) * kSmemBins;
 
@@ -852,21 +909,43 @@ __device__ __forceinline__ void bin_add(unsigned long long* bin, uint64_t X) {
   if ((x2 >> 64) || carry) atomicAdd(bin + 2, (unsigned long long)(x2 >> 64) + carry);
 }
 
-template <bool Trace>
-__device__ __forceinline__ void sample_one(const SamplerArgs& A, const Plan& P, uint64_t W, uint32_t shift,
-                                           uint64_t i, ThreadSums& T, uint32_t* s_err,
-                                           unsigned long long* sbins = nullptr, uint32_t hmin = 0) {
+// The middle-edge draw of sample s from attempt 0's block o (the later
+// attempts run only when it is rejected).
+__device__ __forceinline__ bool middle_draw(const SamplerArgs& A, uint64_t s, const uint4& o, uint64_t W,
+                                            uint64_t* r2) {
+  const uint64_t x = (uint64_t)o.x | ((uint64_t)o.y << 32);
+  *r2 = __umul64hi(x, W);
+  if (x * W >= W) return true;  // accepted whatever the threshold 2^64 mod W
+  uint64_t r;
+  if (!bounded_draw_slow(A.seed, s, W, &r)) return false;
+  *r2 = r;
+  return true;
+}
+
+// Lemire's test and draw for a range below 2^32 (two 32 x 64-bit products;
+// the same result as lemire_accept); false: the low word lies below the
+// range, so the rejection threshold decides.
+__device__ __forceinline__ bool draw32(uint32_t xlo, uint32_t xhi, uint32_t range, uint32_t* out) {
+  const uint64_t p0 = (uint64_t)xlo * range;
+  const uint64_t p1 = (uint64_t)xhi * range + (p0 >> 32);
+  *out = (uint32_t)(p1 >> 32);
+  return (uint32_t)p1 != 0 || (uint32_t)p0 >= range;
+}
+
+// The end edges' draws again with the rejection loop.
+__device__ __noinline__ bool end_draw_slow(uint64_t seed, uint64_t s, bool upper, uint32_t range, uint32_t* out) {
+  uint64_t r;
+  if (!bounded_draw_words(seed, s, 1, upper, range, &r)) return false;
+  *out = (uint32_t)r;
+  return true;
+}
+
+// One sample (Alg. 2, 3) with its middle-edge draw r2: sample index i within
+// the call (id offset + i).
+template <bool Trace, bool Compact>
+__device__ __forceinline__ void sample_one(const SamplerArgs& A, const Plan& P, uint32_t shift, uint64_t i,
+                                           uint64_t r2, ThreadSums& T, unsigned long long* sbins = nullptr, uint32_t hmin = 0) {
   const uint64_t s = A.offset + i;
-  uint64_t r2, r1, r3;
-  const uint2 key = make_uint2((uint32_t)A.seed, (uint32_t)(A.seed >> 32));
-  {
-    const uint4 o = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), 0u, 0u), key);
-    if (!lemire_accept((uint64_t)o.x | ((uint64_t)o.y << 32), W, &r2) &&
-        !bounded_draw_slow(A.seed, s, 0, false, W, &r2)) {
-      T.err |= kErrRng;
-      return;
-    }
-  }
   // middle edge: the unique e with prefix[e] <= r2 < prefix[e + 1]
   const uint32_t b = (uint32_t)(r2 >> shift);
   uint32_t lo = __ldg(A.guide + b), hi = __ldg(A.guide + b + 1);
@@ -874,30 +953,27 @@ __device__ __forceinline__ void sample_one(const SamplerArgs& A, const Plan& P, 
     const uint32_t mid = lo + ((hi - lo + 1) >> 1);
     if (__ldg(A.prefix + mid) <= r2) lo = mid; else hi = mid - 1;
   }
-  if (lo >= A.m) { T.err |= kErrBounds; return; }
-  const EdgeWin e = A.win[lo];
-  const OutEdge me = A.out_e[lo];  // the middle edge (u, v, t)
-  if (e.d1 == 0 || e.d3 == 0) { T.err |= kErrBounds; return; }  // index not built from this prefix
-  // e1 and e3 from the two halves of block 1; a draw over one position is 0
-  // without drawing (a wedge's dummy end, or a window of one edge)
-  r1 = r3 = 0;
-  if (e.d1 > 1 || e.d3 > 1) {
-    const uint4 o = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), 1u, 0u), key);
-    if ((e.d1 > 1 && !lemire_accept((uint64_t)o.x | ((uint64_t)o.y << 32), e.d1, &r1) &&
-         !bounded_draw_slow(A.seed, s, 1, false, e.d1, &r1)) ||
-        (e.d3 > 1 && !lemire_accept((uint64_t)o.z | ((uint64_t)o.w << 32), e.d3, &r3) &&
-         !bounded_draw_slow(A.seed, s, 1, true, e.d3, &r3))) {
-      T.err |= kErrRng;
-      return;
-    }
-  }
-  const uint32_t p1 = e.lo1 + (uint32_t)r1, p3 = e.lo3 + (uint32_t)r3;
-  if (p1 >= A.m || p3 >= A.m) { T.err |= kErrBounds; return; }
+  if (lo >= A.m) { T.fail(kErrBounds); return; }
+  const uint4 e = __ldg(reinterpret_cast<const uint4*>(A.win + lo));  // lo1, d1, lo3, d3
+  const int4 me = __ldg(reinterpret_cast<const int4*>(A.out_e + lo));  // the middle edge (u, v, t)
+  // e1 and e3 from the two halves of block 1, drawn while the two loads are
+  // in flight; a draw over one position is 0 and takes none of them (a
+  // wedge's dummy end, or a window of one edge)
+  const uint4 o = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), 1u, 0u),
+                                make_uint2((uint32_t)A.seed, (uint32_t)(A.seed >> 32)));
+  if (e.y == 0 || e.w == 0) { T.fail(kErrBounds); return; }  // index not built from this prefix
+  uint32_t r1, r3;
+  if (!draw32(o.x, o.y, e.y, &r1) && !end_draw_slow(A.seed, s, false, e.y, &r1)) { T.fail(kErrRng); return; }
+  if (!draw32(o.z, o.w, e.w, &r3) && !end_draw_slow(A.seed, s, true, e.w, &r3)) { T.fail(kErrRng); return; }
+  const uint32_t p1 = e.x + r1, p3 = e.z + r3;
+  if (p1 >= A.m || p3 >= A.m) { T.fail(kErrBounds); return; }
   int32_t up, vp;
-  int64_t t1, t3;
-  end_edge(A, P.alpha1, p1, &up, &t1);
-  end_edge(A, P.alpha3, p3, &vp, &t3);
-  const uint64_t X = check_motif(A, P, up, me.src, me.dst, vp, t1, me.t, t3, s_err, &T.checked);
+  typename SampleTime<Compact>::T t1, t3;
+  end_edge<Compact>(A, P.alpha1, p1, &up, &t1);
+  end_edge<Compact>(A, P.alpha3, p3, &vp, &t3);
+  const typename SampleTime<Compact>::T t2 =
+      SampleTime<Compact>::rel(A, (int64_t)(((uint64_t)(uint32_t)me.w << 32) | (uint32_t)me.z));
+  const uint64_t X = check_motif<Compact>(A, P, up, me.x, me.y, vp, t1, t2, t3, T.s_err, &T.checked);
   if (A.h && X) {  // exact per-h bins of the proposal estimator (the block's own when it has them)
     const uint32_t hv = __ldg(A.h + lo);
     const bool local = sbins && hv - hmin < kSmemBins;  // an h outside the recorded range goes to global
@@ -909,25 +985,453 @@ __device__ __forceinline__ void sample_one(const SamplerArgs& A, const Plan& P, 
     A.trace[4 * i + 2] = p3;
     A.trace[4 * i + 3] = X;
   }
-  const uint64_t nx = T.sx + X;
-  if (nx < T.sx) T.err |= kErrOverflow;
-  T.sx = nx;
-  T.sx2 += (unsigned __int128)X * X;
-  T.hits += X != 0;
+  T.add(X);
+}
+
+// ---------------------------------------------------------------------------
+// Processing order of the samples.  Samples whose middle-edge draws are close
+// share windows, edges and pair lists, and lanes with neighbouring draws run
+// the same searches, so a call's samples are processed in order of their
+// draws.  The draw r = floor(x W / 2^64) is monotone in the 64-bit random
+// word x, so the order needs no weights: it is that of x's high word y, which
+// is uniform over 2^32.  Each chunk's ids are partitioned into nb = nb1 nb2
+// buckets of equal width of y (two passes of nb1 and nb2 buckets, one pass
+// for few buckets), and the sampler's block orders one bucket at a time in
+// shared memory (sample_buckets).
+//
+// The bucket sizes are binomial, so every bucket gets a fixed room of its
+// mean plus eight standard deviations: a tile reserves its run in a bucket
+// with one atomic on the bucket's cursor, and no histogram pass and no scan
+// run before the scatter (a histogram over the draws costs a second Philox
+// block per sample).  Should a bucket ever overflow its room, the order's
+// overflow word is set and the sampler takes the chunk in id order instead:
+// the sums are integers and do not depend on the order.
+//
+// Measured for 1e9 samples of the 300M-edge graph (chunks of 2^28): order
+// passes 7.3 ms (4.1 + 3.2) and sampler 29.5 ms, where two counting passes
+// over 16-bit keys with their histograms and scans took 12.4 ms and the
+// sampler on that order 52.6 ms.  A sampler on the order by 20, 24 or 32 bits
+// of the draw, otherwise unchanged, took 43.5, 38.7 and 39.0 ms: beyond 24
+// bits (the bucket and its bins here) nothing more is gained.
+constexpr int kOrderThreads = 512;
+constexpr int kOrderItems = 16;
+constexpr int kOrderTile = kOrderThreads * kOrderItems;  // 8192
+constexpr uint32_t kOrderMaxDigits = 1024;               // buckets of one pass
+constexpr uint32_t kOrderMaxDigits2 = 512;               // of a second pass: 9 bits carried from the first
+constexpr uint32_t kOrderHeadWords = 64;
+// The buckets fill the sampler's tile of 4096 less two standard deviations
+// (the one in forty that holds more takes a second, small tile).
+constexpr uint32_t kBucketMean = 4096 - 2 * 64;
+static_assert(kOrderTile == 1 << 13 && kOrderMaxDigits == 1 << 10 && kOrderMaxDigits2 == 1 << 9,
+              "digit, position and carry of a staged element are packed into 32 bits");
+
+// Room of a bucket that holds mean elements of a binomial distribution on
+// average.  TC_ORDER_SLACK: standard deviations of room (tests build it small).
+#ifndef TC_ORDER_SLACK
+#define TC_ORDER_SLACK 8
+#endif
+static uint32_t bucket_room(uint64_t count, uint64_t buckets) {
+  const double mean = (double)count / (double)buckets;
+  const double room = mean + TC_ORDER_SLACK * std::sqrt(mean) + 8 * TC_ORDER_SLACK + 1;
+  return (uint32_t)(((uint64_t)room + 31) & ~31ull);
+}
+
+// Layout of an order of count samples: [head: overflow word, next bucket]
+// [cursors of the first pass][bucket sizes][ids by bucket]; scratch: the
+// first pass's ids and carried digits.
+struct OrderPlan {
+  uint32_t nb1, nb2, nb, room1, room;
+  size_t head_bytes, ids_off, bytes;   // order buffer
+  size_t carry_off, scratch_bytes;     // scratch
+};
+
+static OrderPlan order_plan(uint64_t count, uint32_t wave) {
+  OrderPlan L;
+  // whole waves of buckets while they are few (1e6 samples of the 1e7-edge
+  // graph in 456 buckets for 456 resident blocks: 100 us; in 608: 118 us)
+  uint64_t nb = std::max<uint64_t>((count + kBucketMean - 1) / kBucketMean, 1);
+  if (nb < 16ull * wave) nb = (nb + wave - 1) / wave * wave;
+  if (nb <= kOrderMaxDigits) {
+    L.nb1 = 1;
+    L.nb2 = (uint32_t)nb;
+  } else {
+    uint64_t d = 1;
+    while (d * d < nb) d++;
+    L.nb2 = (uint32_t)std::min<uint64_t>(d, kOrderMaxDigits2);
+    L.nb1 = (uint32_t)((nb + L.nb2 - 1) / L.nb2);
+  }
+  L.nb = L.nb1 * L.nb2;
+  L.room = bucket_room(count, L.nb);
+  L.room1 = L.nb1 > 1 ? bucket_room(count, L.nb1) : 0;
+  L.head_bytes = align256(sizeof(uint32_t) * ((size_t)kOrderHeadWords + L.nb1 + L.nb));
+  L.ids_off = L.head_bytes;
+  L.bytes = L.head_bytes + align256(sizeof(uint32_t) * (size_t)L.nb * L.room);
+  L.carry_off = align256(sizeof(uint32_t) * (size_t)L.nb1 * L.room1);
+  L.scratch_bytes = L.nb1 > 1 ? L.carry_off + align256(sizeof(uint16_t) * (size_t)L.nb1 * L.room1) : 0;
+  return L;
+}
+
+size_t order_bytes(uint64_t count, uint32_t wave) { return order_plan(count, wave).bytes; }
+size_t order_scratch_bytes(uint64_t count, uint32_t wave) {
+  return order_plan(count, wave).scratch_bytes;
+}
+
+OrderView order_view(uint64_t count, uint32_t wave, void* order) {
+  const OrderPlan L = order_plan(count, wave);
+  OrderView v;
+  uint32_t* w = (uint32_t*)order;
+  v.head = w;
+  v.sizes = w + kOrderHeadWords + L.nb1;
+  v.ids = (const uint32_t*)((const char*)order + L.ids_off);
+  v.nb = L.nb;
+  v.nb1 = L.nb1;
+  v.nb2 = L.nb2;
+  v.room = L.room;
+  return v;
+}
+
+// Exclusive scan of s_cnt[0 .. 2 kOrderThreads) into s_start, two digits a thread.
+__device__ __forceinline__ void order_scan(const uint32_t* s_cnt, uint32_t* s_start, uint32_t* s_warp) {
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const uint32_t c0 = s_cnt[2 * t], c1 = s_cnt[2 * t + 1];
+  uint32_t inc = c0 + c1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) s_warp[wid] = inc;
+  __syncthreads();
+  uint32_t before = 0;
+#pragma unroll
+  for (int w = 0; w < kOrderThreads / 32; w++) before += w < wid ? s_warp[w] : 0u;
+  const uint32_t ex = before + inc - c0 - c1;
+  s_start[2 * t] = ex;
+  s_start[2 * t + 1] = ex + c0;
+}
+
+// First pass: draws the samples' words y and partitions the ids of a tile of
+// 8192 samples by floor(y nb / 2^32).  TwoLevel: the second pass's digit is
+// carried along.  The tile is staged in shared memory in digit order, so the
+// ids of one digit go out as one run; bound by the Philox block per sample.
+template <bool TwoLevel>
+__global__ void __launch_bounds__(kOrderThreads) k_order_first(uint64_t seed, uint64_t first, uint64_t count,
+                                                              uint32_t nb, uint32_t nb2, uint32_t room,
+                                                              uint32_t* __restrict__ cursor,
+                                                              uint32_t* __restrict__ ids_out,
+                                                              uint16_t* __restrict__ carry_out,
+                                                              uint32_t* __restrict__ overflow) {
+  __shared__ __align__(16) uint32_t s_cnt[kOrderMaxDigits], s_start[kOrderMaxDigits], s_base[kOrderMaxDigits];
+  __shared__ uint32_t s_warp[kOrderThreads / 32];
+  __shared__ uint32_t stage[kOrderTile];
+  const int t = threadIdx.x;
+  s_cnt[t] = s_cnt[t + kOrderThreads] = 0;
+  __syncthreads();
+  const uint64_t base = (uint64_t)blockIdx.x * kOrderTile;
+  const uint32_t n = (uint32_t)(count - base < (uint64_t)kOrderTile ? count - base : (uint64_t)kOrderTile);
+  const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+  uint32_t dk[kOrderItems], rk[kOrderItems];  // (digit << 9 | carried digit), rank in the tile's digit
+#pragma unroll
+  for (int it = 0; it < kOrderItems; it++) {
+    const uint32_t j = (uint32_t)it * kOrderThreads + t;
+    dk[it] = 0xFFFFFFFFu;
+    if (j < n) {
+      const uint64_t s = first + base + j;
+      const uint32_t y = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), 0u, 0u), key).y;
+      const uint32_t d = __umulhi(y, nb);
+      dk[it] = d << 9;
+      if (TwoLevel) dk[it] |= __umulhi(y * nb, nb2);  // digit of the remainder: bucket floor(y nb nb2 / 2^32) in all
+      rk[it] = atomicAdd(&s_cnt[d], 1u);
+    }
+  }
+  __syncthreads();
+  order_scan(s_cnt, s_start, s_warp);
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    const int d = t + h * kOrderThreads;
+    const uint32_t c = s_cnt[d];
+    s_base[d] = c ? atomicAdd(cursor + d, c) : 0u;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kOrderItems; it++)
+    if (dk[it] != 0xFFFFFFFFu)
+      stage[s_start[dk[it] >> 9] + rk[it]] = (dk[it] << 13) | ((uint32_t)it * kOrderThreads + t);
+  __syncthreads();
+  bool over = false;
+  for (uint32_t i = t; i < n; i += kOrderThreads) {
+    const uint32_t e = stage[i], d = e >> 22;
+    const uint32_t pos = s_base[d] + (i - s_start[d]);
+    if (pos < room) {
+      const uint64_t g = (uint64_t)d * room + pos;
+      ids_out[g] = (uint32_t)base + (e & (kOrderTile - 1));
+      if (TwoLevel) carry_out[g] = (uint16_t)((e >> 13) & (kOrderMaxDigits2 - 1));
+    } else {
+      over = true;
+    }
+  }
+  if (over) *overflow = 1;
+}
+
+// Second pass: tile blockIdx.x of the first pass's bucket blockIdx.y, by the carried digit.
+struct OrderSecondShared {
+  uint32_t cnt[kOrderMaxDigits], start[kOrderMaxDigits], base[kOrderMaxDigits];
+  uint32_t warp[kOrderThreads / 32];
+  uint32_t id[kOrderTile];
+  uint16_t d[kOrderTile];
+};
+__global__ void __launch_bounds__(kOrderThreads) k_order_second(const uint32_t* __restrict__ cursor1, uint32_t room1,
+                                                               const uint32_t* __restrict__ ids_in,
+                                                               const uint16_t* __restrict__ carry, uint32_t nb2,
+                                                               uint32_t room, uint32_t* __restrict__ sizes,
+                                                               uint32_t* __restrict__ ids_out,
+                                                               uint32_t* __restrict__ overflow) {
+  extern __shared__ __align__(16) unsigned char order_raw[];
+  OrderSecondShared& S = *reinterpret_cast<OrderSecondShared*>(order_raw);
+  const int t = threadIdx.x;
+  const uint32_t seg = blockIdx.y, size1 = min(cursor1[seg], room1), lo = blockIdx.x * kOrderTile;
+  if (lo >= size1) return;
+  const uint32_t n = min(size1 - lo, (uint32_t)kOrderTile);
+  const uint64_t g0 = (uint64_t)seg * room1 + lo;
+  S.cnt[t] = S.cnt[t + kOrderThreads] = 0;
+  uint32_t id[kOrderItems], dr[kOrderItems];
+#pragma unroll
+  for (int it = 0; it < kOrderItems; it++) {
+    const uint32_t j = (uint32_t)it * kOrderThreads + t;
+    dr[it] = 0xFFFFFFFFu;
+    if (j < n) {
+      id[it] = __ldcs(ids_in + g0 + j);
+      dr[it] = (uint32_t)__ldcs(carry + g0 + j) << 16;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kOrderItems; it++)
+    if (dr[it] != 0xFFFFFFFFu) dr[it] |= atomicAdd(&S.cnt[dr[it] >> 16], 1u);
+  __syncthreads();
+  order_scan(S.cnt, S.start, S.warp);
+  if (t < (int)nb2) {
+    const uint32_t c = S.cnt[t];
+    S.base[t] = c ? atomicAdd(sizes + (uint64_t)seg * nb2 + t, c) : 0u;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kOrderItems; it++)
+    if (dr[it] != 0xFFFFFFFFu) {
+      const uint32_t p = S.start[dr[it] >> 16] + (dr[it] & 0xFFFFu);
+      S.id[p] = id[it];
+      S.d[p] = (uint16_t)(dr[it] >> 16);
+    }
+  __syncthreads();
+  bool over = false;
+  for (uint32_t i = t; i < n; i += kOrderThreads) {
+    const uint32_t d = S.d[i], pos = S.base[d] + (i - S.start[d]);
+    if (pos < room)
+      ids_out[((uint64_t)seg * nb2 + d) * room + pos] = S.id[i];
+    else
+      over = true;
+  }
+  if (over) *overflow = 1;
+}
+
+// Writes the order of samples first .. first + count - 1 (at most
+// kChunkSamples) into order (order_bytes bytes), using only the given scratch
+// of order_scratch_bytes bytes (no allocation).
+tc_status order_samples(uint64_t seed, uint64_t first, uint64_t count, uint32_t wave, void* scratch, void* order,
+                        cudaStream_t st) {
+  static bool attr = false;
+  if (!attr) {
+    TC_CUDA(cudaFuncSetAttribute(k_order_second, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(OrderSecondShared)));
+    attr = true;
+  }
+  const OrderPlan L = order_plan(count, wave);
+  uint32_t* head = (uint32_t*)order;
+  uint32_t* cursor1 = head + kOrderHeadWords;
+  uint32_t* sizes = cursor1 + L.nb1;
+  uint32_t* ids = (uint32_t*)((char*)order + L.ids_off);
+  TC_CUDA(cudaMemsetAsync(order, 0, L.head_bytes, st));
+  const unsigned tiles = (unsigned)((count + kOrderTile - 1) / kOrderTile);
+  if (L.nb1 == 1) {
+    k_order_first<false><<<tiles, kOrderThreads, 0, st>>>(seed, first, count, L.nb2, 0, L.room, sizes, ids, nullptr,
+                                                          head);
+    TC_LAUNCHED(1);
+    TC_CUDA(cudaGetLastError());
+    return TC_OK;
+  }
+  uint32_t* ids1 = (uint32_t*)scratch;
+  uint16_t* carry = (uint16_t*)((char*)scratch + L.carry_off);
+  k_order_first<true><<<tiles, kOrderThreads, 0, st>>>(seed, first, count, L.nb1, L.nb2, L.room1, cursor1, ids1, carry,
+                                                       head);
+  TC_LAUNCHED(1);
+  TC_CUDA(cudaGetLastError());
+  const dim3 grid((L.room1 + kOrderTile - 1) / kOrderTile, L.nb1);
+  k_order_second<<<grid, kOrderThreads, sizeof(OrderSecondShared), st>>>(cursor1, L.room1, ids1, carry, L.nb2, L.room,
+                                                                         sizes, ids, head);
+  TC_LAUNCHED(1);
+  TC_CUDA(cudaGetLastError());
+  return TC_OK;
+}
+
+// ---------------------------------------------------------------------------
+// The sampler's block works through buckets of samples: it draws r for a
+// tile of up to 8 BS of the bucket's samples, orders them by the finer bits
+// of their draws in shared memory (a counting sort over 2 BS bins, ranks from
+// shared-memory atomics), and its warps then take them in that order, 32 at a
+// time from a counter, so that a warp's samples lie on a few neighbouring
+// middle edges: their CDF searches take the same steps and their loads fall
+// in the same sectors.  Shared memory is kept small, because the searches
+// live from the L1 that it leaves: a sample takes its id and the low 32 bits
+// of r - r0, r0 the smallest draw of the bucket; where the draws of a bucket
+// span more than 32 bits, r is drawn again from the id.
+//
+// Bound by latency and issue together (ncu, 1e8 samples of the 20M-edge
+// graph: issue slots 50% busy, long-scoreboard stalls 13 of 24 cycles, DRAM
+// 31%), so by resident warps: 40 registers, which hold 48 warps per SM, spill
+// a little and still take 30 ms per 1e9 samples where 64 registers took 38.7
+// and 32 registers 41; 12 KB more shared memory per block (an SM's L1 falls
+// from 92 to 60 KB) cost 30%, and tiles of 2048 samples 10%.
+constexpr int kBucketItems = 8;
+template <int BS>
+struct TileShared {
+  uint32_t id[kBucketItems * BS];
+  uint32_t r[kBucketItems * BS];
+  uint2 cnt[BS];  // 2 BS bins, later the bins' starts
+  uint32_t warp[BS / 32];
+  unsigned long long r0;  // the bucket's smallest draw
+  uint32_t next;          // next place to take
+};
+constexpr uint32_t kDrawAgain = 0xFFFFFFFFu;  // instead of r - r0: r is drawn from the id
+
+
+template <int BS, bool Trace, bool Compact>
+__device__ __forceinline__ void sample_bucket(const SamplerArgs& A, const Plan& P, uint64_t W, uint32_t shift,
+                                              uint32_t bucket, TileShared<BS>& S, ThreadSums& T,
+                                              unsigned long long* sbins, uint32_t hmin) {
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const uint32_t size = min(A.ord.sizes[bucket], A.ord.room);
+  const uint2 key = make_uint2((uint32_t)A.seed, (uint32_t)(A.seed >> 32));
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(S.cnt);
+  // the bucket's words y lie in a range of 2^32 / nb, its draws in one of
+  // W / nb + W / 2^32 + 1 (nb <= 2^20 buckets)
+  const bool wide = W >= (uint64_t)A.ord.nb << 31;
+  for (uint32_t base = 0; base < size; base += kBucketItems * BS) {
+    const uint32_t n = min(size - base, (uint32_t)(kBucketItems * BS));
+    const uint32_t* ids = A.ord.ids + (uint64_t)bucket * A.ord.room + base;
+    S.cnt[t] = make_uint2(0, 0);
+    if (t == 0) {
+      S.next = 0;
+      const uint64_t y0 = (((uint64_t)bucket << 32) + A.ord.nb - 1) / A.ord.nb;  // the bucket's first word
+      S.r0 = __umul64hi(y0 << 32, W);
+    }
+    __syncthreads();
+    uint32_t br[kBucketItems];  // bin and rank
+#pragma unroll
+    for (int it = 0; it < kBucketItems; it++) {
+      const uint32_t j = (uint32_t)it * BS + t;
+      br[it] = 0xFFFFFFFFu;
+      if (j < n) {
+        const uint32_t id = __ldcs(ids + j);
+        const uint64_t s = A.offset + A.chunk_base + id;
+        const uint4 o = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), 0u, 0u), key);
+        const uint64_t x = (uint64_t)o.x | ((uint64_t)o.y << 32);
+        S.id[j] = id;
+        // (x W mod 2^64 < W: attempt 0 may be rejected)
+        S.r[j] = wide || x * W < W ? kDrawAgain : (uint32_t)(__umul64hi(x, W) - S.r0);
+        const uint32_t bin = __umulhi(o.y * A.ord.nb, 2 * BS);  // by the position inside the bucket
+        br[it] = (bin << 16) | atomicAdd(&cnt[bin], 1u);
+      }
+    }
+    __syncthreads();
+    {  // exclusive scan of the bins, two a thread
+      const uint2 c = S.cnt[t];
+      uint32_t inc = c.x + c.y;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      if (lane == 31) S.warp[wid] = inc;
+      __syncthreads();
+      uint32_t ex = inc - c.x - c.y;
+      for (int w = 0; w < wid; w++) ex += S.warp[w];
+      S.cnt[t] = make_uint2(ex, ex + c.x);
+    }
+    uint32_t id[kBucketItems], r[kBucketItems];
+#pragma unroll
+    for (int it = 0; it < kBucketItems; it++) {
+      id[it] = S.id[it * BS + t];
+      r[it] = S.r[it * BS + t];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kBucketItems; it++)
+      if (br[it] != 0xFFFFFFFFu) {
+        const uint32_t p = cnt[br[it] >> 16] + (br[it] & 0xFFFFu);
+        S.id[p] = id[it];
+        S.r[p] = r[it];
+      }
+    __syncthreads();
+    const uint64_t r0 = S.r0;
+    for (;;) {
+      uint32_t p = 0;
+      if (lane == 0) p = atomicAdd(&S.next, 32u);
+      p = __shfl_sync(0xffffffffu, p, 0);
+      if (p >= n) break;
+      p += lane;
+      if (p < n) {
+        const uint64_t i = A.chunk_base + S.id[p];
+        uint64_t r2 = r0 + S.r[p];
+        if (S.r[p] == kDrawAgain && !bounded_draw_slow(A.seed, A.offset + i, W, &r2))
+          T.fail(kErrRng);
+        else
+          sample_one<Trace, Compact>(A, P, shift, i, r2, T, sbins, hmin);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Samples [lo, hi) of the chunk in id order.
+template <int BS, bool Trace, bool Compact>
+__device__ __forceinline__ void sample_ids(const SamplerArgs& A, const Plan& P, uint64_t W, uint32_t shift,
+                                           uint64_t lo, uint64_t hi, uint64_t stride, ThreadSums& T,
+                                           unsigned long long* sbins, uint32_t hmin) {
+  const uint2 key = make_uint2((uint32_t)A.seed, (uint32_t)(A.seed >> 32));
+#pragma unroll 1
+  for (uint64_t j = lo; j < hi; j += stride) {
+    const uint64_t i = A.chunk_base + j, s = A.offset + i;
+    const uint4 o = philox4x32_10(make_uint4((uint32_t)s, (uint32_t)(s >> 32), 0u, 0u), key);
+    uint64_t r2;
+    if (middle_draw(A, s, o, W, &r2))
+      sample_one<Trace, Compact>(A, P, shift, i, r2, T, sbins, hmin);
+    else
+      T.fail(kErrRng);
+  }
 }
 
 // Proposal mode: a block accumulates the per-h bins of its samples in
 // shared memory (kSmemBins consecutive h values from the proposal's
 // smallest h) and adds them to the global bins once at its end, instead of
 // one global atomic per hit on a few hot bins.
-template <bool Trace>
-__global__ void __launch_bounds__(256, TC_SAMPLE_MIN_BLOCKS) k_sample(const __grid_constant__ SamplerArgs A,
-                                                const __grid_constant__ Plan P) {
-  extern __shared__ unsigned long long s_bins[];  // kSmemBinBytes in proposal mode, else none
+//
+// The blocks take the order's buckets one after the other from a counter, and
+// a block's warps its samples: buckets on hub edges cost more than others (a
+// fixed share per block left the slowest SM 16% behind the mean), and so do
+// samples with long lists (with list_count_two, 5e6 samples of a
+// motif with two lists in its last gap went from 1.55 to 0.40 ms).
+constexpr int kSampleThreads = 512;
+template <bool Trace, bool Compact>
+__global__ void __launch_bounds__(kSampleThreads, TC_SAMPLE_MIN_BLOCKS) k_sample(const __grid_constant__ SamplerArgs A,
+                                                                                const __grid_constant__ Plan P) {
+  extern __shared__ __align__(16) unsigned char sample_raw[];  // TileShared (ordered samples), then the bins (proposal mode)
+  TileShared<kSampleThreads>& S = *reinterpret_cast<TileShared<kSampleThreads>*>(sample_raw);
+  unsigned long long* s_bins =
+      reinterpret_cast<unsigned long long*>(sample_raw + (A.ord.nb ? sizeof(TileShared<kSampleThreads>) : 0));
   const IndexHeader* H = A.hdr;
   const uint64_t W = H->W;
   const uint32_t shift = H->shift;
-  __shared__ uint32_t s_err;
+  __shared__ uint32_t s_err, s_item;
   __shared__ unsigned long long s_x, s_x2lo, s_x2hi, s_hits, s_checked;
   if (threadIdx.x == 0) {
     s_err = 0;
@@ -947,11 +1451,21 @@ __global__ void __launch_bounds__(256, TC_SAMPLE_MIN_BLOCKS) k_sample(const __gr
     if (threadIdx.x == 0) atomicOr(&A.sums->err, bad);
     return;
   }
-  ThreadSums T;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < A.count && W; j += stride) {
-    const uint64_t i = A.chunk_base + (A.order ? __ldg(A.order + j) : j);  // sample index within the call
-    sample_one<Trace>(A, P, W, shift, i, T, &s_err, local_bins ? s_bins : nullptr, hmin);
+  ThreadSums T(&s_err);
+  unsigned long long* bins = local_bins ? s_bins : nullptr;
+  if (W && A.ord.nb && A.ord.head[0] == 0) {
+    for (;;) {
+      if (threadIdx.x == 0) s_item = atomicAdd(A.ord.head + 1, 1u);
+      __syncthreads();
+      const uint32_t item = s_item;
+      if (item >= A.ord.nb) break;
+      sample_bucket<kSampleThreads, Trace, Compact>(A, P, W, shift, item, S, T, bins, hmin);
+      __syncthreads();
+    }
+  } else if (W) {  // id order: few samples, or an order that overflowed
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    sample_ids<kSampleThreads, Trace, Compact>(A, P, W, shift, (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, A.count,
+                                               stride, T, bins, hmin);
   }
   if (local_bins) {
     __syncthreads();
@@ -965,275 +1479,7 @@ __global__ void __launch_bounds__(256, TC_SAMPLE_MIN_BLOCKS) k_sample(const __gr
       if (hi || carry) atomicAdd(g + 2, hi + carry);
     }
   }
-  block_commit(A.sums, W, T.sx, T.sx2, T.hits, T.checked, T.err, s_err, s_x, s_x2lo, s_x2hi, s_hits, s_checked);
-}
-
-// Processing order of the samples.  Samples whose middle-edge draws r are
-// close share records, windows and pair lists, so each chunk of samples is
-// put in order of the top 16 bits of r by a two-pass most-significant-digit
-// counting sort: pass A partitions the samples by the high byte of the key
-// into 256 segments, pass B orders each segment by the low byte.  The order
-// of samples with equal keys is free, so ranks inside a tile come from
-// shared-memory atomics; tiles are staged in shared memory in digit order so
-// that global writes form contiguous runs.  The first pass draws r once per
-// sample and stores its 16-bit key.  Integer sums do not depend on the order.
-constexpr int kBuckets = 256;
-constexpr int kBucketItems = 16;
-constexpr int kBucketTile = 256 * kBucketItems;
-
-struct SegInfo {          // pass-B tiling of the 256 segments of pass A
-  uint32_t start[kBuckets + 1];      // first element of each segment
-  uint32_t ntiles[kBuckets];         // tiles of each segment
-  uint32_t tile_base[kBuckets + 1];  // first tile of each segment
-};
-
-// Pass A histogram: draws the keys (writing them in id order) and counts
-// their high bytes; hist[d * tiles + tile].
-__global__ void __launch_bounds__(256) k_key_hist(const IndexHeader* __restrict__ H, uint64_t seed, uint64_t first,
-                                                  uint64_t count, uint16_t* __restrict__ keys,
-                                                  uint32_t* __restrict__ hist, uint32_t tiles) {
-  __shared__ uint32_t cnt[kBuckets];
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const uint64_t W = H->W;
-  const int wbits = W > 1 ? 64 - __clzll(W - 1) : 0;
-  const int drop = wbits > 16 ? wbits - 16 : 0;
-  const uint64_t base = (uint64_t)blockIdx.x * kBucketTile;
-#pragma unroll 4
-  for (int it = 0; it < kBucketItems; it++) {
-    const uint64_t j = base + (uint64_t)it * 256 + threadIdx.x;
-    if (j < count) {
-      uint64_t r = 0;
-      if (W) bounded_draw(seed, first + j, 0, W, &r);  // a failed draw is flagged by the sampler
-      const uint32_t key = (uint32_t)(r >> drop);
-      keys[j] = (uint16_t)key;
-      atomicAdd(&cnt[key >> 8], 1u);
-    }
-  }
-  __syncthreads();
-  hist[(uint64_t)threadIdx.x * tiles + blockIdx.x] = cnt[threadIdx.x];
-}
-
-// Scatter the elements [lo, hi) of one tile by digit (key >> shift) & 255 to
-// out_base[d] + rank, staging the tile in shared memory in digit order.
-// ids_in == NULL means the element's own position.
-__device__ __forceinline__ void tile_scatter(uint32_t lo, uint32_t hi, const uint16_t* __restrict__ keys_in,
-                                             const uint32_t* __restrict__ ids_in, int shift,
-                                             const uint32_t* s_out_base, uint16_t* __restrict__ keys_out,
-                                             uint32_t* __restrict__ ids_out, uint32_t* cnt, uint32_t* start,
-                                             uint32_t* warp_tot, uint32_t* stage, uint16_t* stage_k) {
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  // key (16 bits) and rank within the tile (< kBucketTile) packed in one
-  // register per item; the ids are loaded up front with the keys
-  uint32_t kr[kBucketItems], id[kBucketItems];
-#pragma unroll
-  for (int it = 0; it < kBucketItems; it++) {
-    const uint32_t j = lo + (uint32_t)it * 256 + threadIdx.x;
-    kr[it] = 0xFFFFFFFFu;
-    if (j < hi) {
-      kr[it] = (uint32_t)__ldg(keys_in + j) << 16;
-      id[it] = ids_in ? __ldg(ids_in + j) : j;
-    }
-  }
-#pragma unroll
-  for (int it = 0; it < kBucketItems; it++)
-    if (kr[it] != 0xFFFFFFFFu) kr[it] |= atomicAdd(&cnt[((kr[it] >> 16) >> shift) & 255u], 1u);
-  __syncthreads();
-  {  // exclusive scan of the tile's digit counts
-    const uint32_t v = cnt[threadIdx.x];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t inc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) warp_tot[wid] = inc;
-    __syncthreads();
-    uint32_t before = 0;
-    for (int w = 0; w < wid; w++) before += warp_tot[w];
-    start[threadIdx.x] = before + inc - v;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int it = 0; it < kBucketItems; it++) {
-    if (kr[it] != 0xFFFFFFFFu) {
-      const uint32_t key = kr[it] >> 16;
-      const uint32_t p = start[(key >> shift) & 255u] + (kr[it] & 0xFFFFu);
-      stage[p] = id[it];
-      stage_k[p] = (uint16_t)key;
-    }
-  }
-  __syncthreads();
-  const uint32_t n = hi - lo;
-  for (uint32_t i = threadIdx.x; i < n; i += 256) {
-    const uint32_t kk = stage_k[i];
-    const uint32_t d = (kk >> shift) & 255u;
-    const uint32_t g = s_out_base[d] + (i - start[d]);
-    ids_out[g] = stage[i];
-    if (keys_out) keys_out[g] = (uint16_t)kk;
-  }
-}
-
-// Pass A scatter: tile t of the chunk, by the high byte.
-__global__ void __launch_bounds__(256, 6) k_key_scatter_a(uint64_t count, const uint16_t* __restrict__ keys,
-                                                       const uint32_t* __restrict__ offs, uint32_t tiles,
-                                                       uint16_t* __restrict__ keys_out,
-                                                       uint32_t* __restrict__ ids_out) {
-  __shared__ uint32_t cnt[kBuckets], start[kBuckets], base_s[kBuckets], warp_tot[8];
-  __shared__ uint32_t stage[kBucketTile];
-  __shared__ uint16_t stage_k[kBucketTile];
-  base_s[threadIdx.x] = offs[(uint64_t)threadIdx.x * tiles + blockIdx.x];
-  const uint64_t lo = (uint64_t)blockIdx.x * kBucketTile;
-  const uint64_t hi = lo + kBucketTile < count ? lo + kBucketTile : count;
-  tile_scatter((uint32_t)lo, (uint32_t)hi, keys, nullptr, 8, base_s, keys_out, ids_out, cnt, start, warp_tot, stage,
-               stage_k);
-}
-
-// Segment sizes from the scanned pass-A histogram and the pass-B tiling.
-__global__ void k_seg_info(const uint32_t* __restrict__ offs, uint32_t tiles, uint64_t count, SegInfo* info) {
-  __shared__ uint32_t nt[kBuckets + 1];
-  const int d = threadIdx.x;
-  const uint32_t s0 = offs[(uint64_t)d * tiles];
-  const uint32_t s1 = d + 1 < kBuckets ? offs[(uint64_t)(d + 1) * tiles] : (uint32_t)count;
-  info->start[d] = s0;
-  if (d == kBuckets - 1) info->start[kBuckets] = (uint32_t)count;
-  nt[d] = (s1 - s0 + kBucketTile - 1) / kBucketTile;
-  info->ntiles[d] = nt[d];
-  __syncthreads();
-  if (d == 0) {
-    uint32_t run = 0;
-    for (int i = 0; i < kBuckets; i++) {
-      info->tile_base[i] = run;
-      run += nt[i];
-    }
-    info->tile_base[kBuckets] = run;
-  }
-}
-
-// Segment and tile of pass-B block b (false past the last tile).
-__device__ __forceinline__ bool seg_tile(const SegInfo* info, uint32_t b, uint32_t* seg, uint32_t* t) {
-  if (b >= info->tile_base[kBuckets]) return false;
-  uint32_t lo = 0, hi = kBuckets - 1;  // last segment with tile_base <= b
-  while (lo < hi) {
-    const uint32_t mid = (lo + hi + 1) >> 1;
-    if (info->tile_base[mid] <= b) lo = mid; else hi = mid - 1;
-  }
-  *seg = lo;
-  *t = b - info->tile_base[lo];
-  return true;
-}
-
-// Pass B: histogram of the low byte per (segment, digit, tile) at
-// tile_base[s] * 256 + d * ntiles[s] + t, so that one flat exclusive scan
-// gives every element's final position.
-__global__ void __launch_bounds__(256) k_key_hist_b(const uint16_t* __restrict__ keys, const SegInfo* __restrict__ info,
-                                                    uint32_t* __restrict__ hist) {
-  __shared__ uint32_t cnt[kBuckets];
-  uint32_t seg, t;
-  if (!seg_tile(info, blockIdx.x, &seg, &t)) return;
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const uint32_t lo = info->start[seg] + t * kBucketTile;
-  const uint32_t end = info->start[seg + 1];
-  const uint32_t hi = lo + kBucketTile < end ? lo + kBucketTile : end;
-  for (uint32_t j = lo + threadIdx.x; j < hi; j += 256) atomicAdd(&cnt[__ldg(keys + j) & 255u], 1u);
-  __syncthreads();
-  hist[(uint64_t)info->tile_base[seg] * kBuckets + (uint64_t)threadIdx.x * info->ntiles[seg] + t] = cnt[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(256, 5) k_key_scatter_b(const uint16_t* __restrict__ keys,
-                                                       const uint32_t* __restrict__ ids,
-                                                       const SegInfo* __restrict__ info,
-                                                       const uint32_t* __restrict__ offs,
-                                                       uint32_t* __restrict__ ids_out) {
-  __shared__ uint32_t cnt[kBuckets], start[kBuckets], base_s[kBuckets], warp_tot[8];
-  __shared__ uint32_t stage[kBucketTile];
-  __shared__ uint16_t stage_k[kBucketTile];
-  uint32_t seg, t;
-  if (!seg_tile(info, blockIdx.x, &seg, &t)) return;
-  base_s[threadIdx.x] = offs[(uint64_t)info->tile_base[seg] * kBuckets + (uint64_t)threadIdx.x * info->ntiles[seg] + t];
-  const uint32_t lo = info->start[seg] + t * kBucketTile;
-  const uint32_t end = info->start[seg + 1];
-  const uint32_t hi = lo + kBucketTile < end ? lo + kBucketTile : end;
-  tile_scatter(lo, hi, keys, ids, 0, base_s, nullptr, ids_out, cnt, start, warp_tot, stage, stage_k);
-}
-
-// Scratch layout of sort_sample_ids for count samples: ids after pass A,
-// keys in id order and after pass A, the digit histogram, the segment tiling
-// and the histogram scan's tile sums.
-struct SortScratch {
-  uint32_t tiles, tiles_b;
-  size_t ids_a, keys_0, keys_a, hist, info, scan, bytes;  // byte offsets; total
-  uint64_t scan_words;
-};
-
-static SortScratch sort_scratch(uint64_t count) {
-  SortScratch L;
-  L.tiles = (uint32_t)((count + kBucketTile - 1) / kBucketTile);
-  L.tiles_b = L.tiles + kBuckets;
-  const uint64_t cap = (uint64_t)L.tiles * kBucketTile;
-  L.scan_words = scan_u64_scratch_words((uint64_t)kBuckets * L.tiles_b) + 1;
-  size_t p = 0;
-  L.ids_a = p;
-  p += align256(4 * cap);
-  L.keys_0 = p;
-  p += align256(2 * cap);
-  L.keys_a = p;
-  p += align256(2 * cap);
-  L.hist = p;
-  p += align256(4 * ((uint64_t)kBuckets * L.tiles_b + 1));
-  L.info = p;
-  p += align256(sizeof(SegInfo));
-  L.scan = p;
-  p += align256(4 * L.scan_words);
-  L.bytes = p;
-  return L;
-}
-
-size_t sort_scratch_bytes(uint64_t count) { return sort_scratch(count).bytes; }
-
-// Writes the indices 0..count-1 of samples first..first+count-1 into order
-// in key order (top 16 bits of each sample's middle-edge draw), using only
-// the given scratch of sort_scratch_bytes(count) bytes (no allocation).
-tc_status sort_sample_ids(const IndexHeader* hdr, uint64_t seed, uint64_t first, uint64_t count, void* scratch,
-                          uint32_t* order, cudaStream_t st) {
-  const SortScratch L = sort_scratch(count);
-  const uint32_t tiles = L.tiles, tiles_b = L.tiles_b;
-  char* base = (char*)scratch;
-  uint32_t* ids_a = (uint32_t*)(base + L.ids_a);
-  uint16_t* keys_0 = (uint16_t*)(base + L.keys_0);
-  uint16_t* keys_a = (uint16_t*)(base + L.keys_a);
-  uint32_t* hist = (uint32_t*)(base + L.hist);
-  SegInfo* info = (SegInfo*)(base + L.info);
-  uint32_t* scan_scratch = (uint32_t*)(base + L.scan);
-  const uint64_t scan_words = L.scan_words;
-  tc_status s = TC_OK;
-  auto ok = [&](const char* what) {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) s = cuda_status(e, what);
-    return s == TC_OK;
-  };
-  k_key_hist<<<tiles, 256, 0, st>>>(hdr, seed, first, count, keys_0, hist, tiles);
-  TC_LAUNCHED(1);
-  if (!ok("k_key_hist")) return s;
-  TC_TRY(scan_u32_in_scratch(hist, hist, (uint64_t)kBuckets * tiles, scan_scratch, scan_words, st));
-  k_key_scatter_a<<<tiles, 256, 0, st>>>(count, keys_0, hist, tiles, keys_a, ids_a);
-  TC_LAUNCHED(1);
-  if (!ok("k_key_scatter_a")) return s;
-  k_seg_info<<<1, kBuckets, 0, st>>>(hist, tiles, count, info);
-  TC_LAUNCHED(1);
-  if (!ok("k_seg_info")) return s;
-  TC_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)kBuckets * tiles_b, st));
-  k_key_hist_b<<<tiles_b, 256, 0, st>>>(keys_a, info, hist);
-  TC_LAUNCHED(1);
-  if (!ok("k_key_hist_b")) return s;
-  TC_TRY(scan_u32_in_scratch(hist, hist, (uint64_t)kBuckets * tiles_b, scan_scratch, scan_words, st));
-  k_key_scatter_b<<<tiles_b, 256, 0, st>>>(keys_a, ids_a, info, hist, order);
-  TC_LAUNCHED(1);
-  ok("k_key_scatter_b");
-  return s;
+  block_commit(A.sums, W, T.sx, T.sx2, T.hits, T.checked, 0, s_err, s_x, s_x2lo, s_x2hi, s_hits, s_checked);
 }
 
 // Diagnostic timing by phase (tc_set_timing): event pairs around the
@@ -1308,9 +1554,9 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
   A.win = v.win;
   A.guide = v.guide;
   A.k = k;
-  A.order = nullptr;
   A.chunk_base = 0;
   A.count = k;
+  A.ord = OrderView{};
   A.m = (uint32_t)m;
   A.seed = seed;
   A.offset = offset;
@@ -1322,54 +1568,59 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
   A.bins = bins;
   A.hrange = h ? (const uint32_t*)((const char*)qindex + kProposalRangeOffset) : nullptr;
   A.rec_hdr = rec_hdr;
-  static int blocks_per_sm[2] = {0, 0};
-  const int ti = trace ? 1 : 0;
+  const bool compact = A.pair_t32 != nullptr;
+  auto kernel = trace ? (compact ? k_sample<true, true> : k_sample<true, false>)
+                      : (compact ? k_sample<false, true> : k_sample<false, false>);
+  constexpr size_t kTileBytes = sizeof(TileShared<kSampleThreads>);
+  static int blocks_per_sm[4] = {0, 0, 0, 0};
+  const int ti = (trace ? 2 : 0) + (compact ? 1 : 0);
   if (!blocks_per_sm[ti]) {
     int b = 0;
-    if (trace)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample<true>, 256, kSmemBinBytes);
-    else
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample<false>, 256, kSmemBinBytes);
+    TC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kTileBytes + kSmemBinBytes)));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kSampleThreads, kTileBytes + kSmemBinBytes);
     blocks_per_sm[ti] = b > 0 ? b : 1;
   }
   const uint64_t max_blocks = (uint64_t)num_sms() * blocks_per_sm[ti];
-  auto run = [&](const uint32_t* order, uint64_t base, uint64_t count) -> tc_status {
-    A.order = order;
+  auto run = [&](const OrderView& ord, uint64_t base, uint64_t count) -> tc_status {
+    A.ord = ord;
     A.chunk_base = base;
     A.count = count;
     uint64_t blocks = max_blocks;
-    const uint64_t need = (count + 255) / 256;
+    const uint64_t need = ord.nb ? ord.nb : (count + kSampleThreads - 1) / kSampleThreads;
     if (need < blocks) blocks = need ? need : 1;
-    const size_t dyn = h ? kSmemBinBytes : 0;
-    if (trace)
-      k_sample<true><<<(unsigned)blocks, 256, dyn, st>>>(A, plan);
-    else
-      k_sample<false><<<(unsigned)blocks, 256, dyn, st>>>(A, plan);
+    const size_t dyn = (ord.nb ? kTileBytes : 0) + (h ? kSmemBinBytes : 0);
+    kernel<<<(unsigned)blocks, kSampleThreads, dyn, st>>>(A, plan);
     TC_LAUNCHED(1);
     TC_CUDA(cudaGetLastError());
     return TC_OK;
   };
   PhaseTimer timer(TC_PHASE_SAMPLE, st), sort_timer(TC_PHASE_ORDER, st);
-  if (k < kSortedMinSamples) {
+  if (k < kOrderedMinSamples) {
     timer.start();
-    tc_status s = run(nullptr, 0, k);
+    tc_status s = run(OrderView{}, 0, k);
     timer.stop();
     return s;
   }
-  // samples in chunks; each chunk is put in key order first
+  // samples in chunks, each with an order of its own
   const uint64_t chunk = k < kChunkSamples ? k : kChunkSamples;
-  const size_t sbytes = sort_scratch_bytes(chunk);
+  const uint32_t wave = (uint32_t)max_blocks;
+  const size_t sbytes = order_scratch_bytes(chunk, wave);
   char* buf = nullptr;
-  TC_CUDA(pool_malloc(&buf, sbytes + 4 * chunk, st));
-  uint32_t* order = (uint32_t*)(buf + sbytes);
+  // the last chunk is smaller than the others, but its order may hold more rounding
+  const uint64_t tail = k % chunk;
+  const size_t obytes = std::max(order_bytes(chunk, wave), tail ? order_bytes(tail, wave) : (size_t)0);
+  const size_t scratch = std::max(sbytes, tail ? order_scratch_bytes(tail, wave) : (size_t)0);
+  TC_CUDA(pool_malloc(&buf, scratch + obytes, st));
+  void* order = buf + scratch;
   tc_status s = TC_OK;
   for (uint64_t base = 0; base < k && s == TC_OK; base += chunk) {
     const uint64_t count = (k - base) < chunk ? (k - base) : chunk;
     sort_timer.start();
-    s = sort_sample_ids(v.hdr, seed, offset + base, count, buf, order, st);
+    s = order_samples(seed, offset + base, count, wave, buf, order, st);
     sort_timer.stop();
     timer.start();
-    if (s == TC_OK) s = run(order, base, count);
+    if (s == TC_OK) s = run(order_view(count, wave, order), base, count);
     timer.stop();
   }
   cudaFreeAsync(buf, st);
@@ -1398,11 +1649,12 @@ tc_status launch_path_sum(const tc_graph* g, const Plan& plan, int64_t delta, co
   A.graph_id = g->id;
   A.sums = d_sums;
   int bps = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_path_sum, 256, 0);
+  auto kernel = A.pair_t32 ? k_path_sum<true> : k_path_sum<false>;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, 256, 0);
   uint64_t blocks = (uint64_t)num_sms() * (bps > 0 ? bps : 1);
   const uint64_t need = (W + 255) / 256;
   if (need < blocks) blocks = need ? need : 1;
-  k_path_sum<<<(unsigned)blocks, 256, 0, st>>>(A, plan, 0, W);
+  kernel<<<(unsigned)blocks, 256, 0, st>>>(A, plan, 0, W);
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());
   return TC_OK;
@@ -1424,7 +1676,8 @@ static_assert(sizeof(BatchQuery) <= kBatchQueryBytes, "batch record too large");
 static_assert(kBatchQueryBytes % 16 == 0, "batch record must be whole 16-byte words");
 
 void batch_query_record(void* h_rec, const tc_graph* g, const Plan& plan, int64_t delta, const uint64_t* prefix,
-                        const void* index, uint64_t k, uint64_t seed, uint64_t offset, const uint32_t* order) {
+                        const void* index, uint64_t seed, uint64_t offset, uint64_t chunk_base, uint64_t count,
+                        void* order, SampleSums* sums) {
   std::memset(h_rec, 0, kBatchQueryBytes);
   BatchQuery* Q = (BatchQuery*)h_rec;
   const uint64_t m = (uint64_t)g->m;
@@ -1441,24 +1694,44 @@ void batch_query_record(void* h_rec, const tc_graph* g, const Plan& plan, int64_
   A.hdr = v.hdr;
   A.win = v.win;
   A.guide = v.guide;
-  A.k = k;
+  A.k = count;
   A.seed = seed;
   A.offset = offset;
-  A.order = order;
-  A.chunk_base = 0;
-  A.count = k;
+  A.chunk_base = chunk_base;
+  A.count = count;
+  if (order) A.ord = order_view(count, 1, order);
   A.m = (uint32_t)m;
   A.delta = delta;
   A.graph_id = g->id;
+  A.sums = sums;
   Q->P = plan;
 }
 
-template <int BS>
-__global__ void __launch_bounds__(BS, (256 * TC_SAMPLE_MIN_BLOCKS) / BS)
+static uint32_t batch_record_group(const void* h_rec, uint32_t tile) {
+  const SamplerArgs& A = ((const BatchQuery*)h_rec)->A;
+  if (!A.ord.nb) return 0;
+  const uint64_t group = (uint64_t)tile * A.ord.nb / (A.count ? A.count : 1);
+  return (uint32_t)(group ? group : 1);
+}
+
+uint64_t batch_record_items(const void* h_rec, uint32_t tile) {
+  const SamplerArgs& A = ((const BatchQuery*)h_rec)->A;
+  const uint32_t group = batch_record_group(h_rec, tile);
+  return group ? (A.ord.nb + group - 1) / group : (A.count + tile - 1) / tile;
+}
+
+// Compact: the records of graphs with 32-bit list times, else those with
+// 64-bit times only (a kernel each, so that neither pays for the other's
+// registers); a record's items are buckets [j group, (j + 1) group) of its
+// order, or tiles of its ids when it has no order or one that overflowed.
+template <int BS, bool Compact>
+__global__ void __launch_bounds__(BS, (512 * TC_SAMPLE_MIN_BLOCKS) / BS)
     k_sample_batch(const char* __restrict__ records, const uint64_t* __restrict__ tile_begin, uint32_t nq,
-                   uint32_t tile, unsigned long long* __restrict__ next_item, SampleSums* __restrict__ sums) {
+                   uint32_t tile, unsigned long long* __restrict__ next_item) {
+  extern __shared__ __align__(16) unsigned char batch_raw[];
+  TileShared<BS>& S = *reinterpret_cast<TileShared<BS>*>(batch_raw);
   __shared__ BatchQuery s_q;
-  __shared__ unsigned long long s_item;
+  __shared__ unsigned long long s_j;
   __shared__ uint32_t s_query;
   __shared__ uint32_t s_err;
   __shared__ unsigned long long s_x, s_x2lo, s_x2hi, s_hits, s_checked;
@@ -1466,37 +1739,36 @@ __global__ void __launch_bounds__(BS, (256 * TC_SAMPLE_MIN_BLOCKS) / BS)
     s_err = 0;
     s_x = s_x2lo = s_x2hi = s_hits = s_checked = 0;
   }
-  const uint64_t total = tile_begin[nq];
-  uint32_t cur = 0xFFFFFFFFu, bad = 0, shift = 0;
-  uint64_t W = 0;
-  ThreadSums T;
+  uint32_t cur = 0xFFFFFFFFu;
+  bool bad = false;
+  ThreadSums T(&s_err);
   for (;;) {
     if (threadIdx.x == 0) {
       const unsigned long long item = atomicAdd(next_item, 1ull);
       uint32_t q = nq;
-      if (item < total) {  // the last query whose first item is <= item
+      if (item < tile_begin[nq]) {  // the last record whose first item is <= item
         uint32_t lo = 0, hi = nq - 1;
         while (lo < hi) {
           const uint32_t mid = (lo + hi + 1) >> 1;
           if (tile_begin[mid] <= item) lo = mid; else hi = mid - 1;
         }
         q = lo;
+        s_j = item - tile_begin[q];
       }
-      s_item = item;
       s_query = q;
     }
     __syncthreads();
-    const uint64_t item = s_item;
     const uint32_t q = s_query;
     if (q != cur) {  // block-uniform
       if (cur != 0xFFFFFFFFu && !bad) {
-        block_commit(sums + cur, W, T.sx, T.sx2, T.hits, T.checked, T.err, s_err, s_x, s_x2lo, s_x2hi, s_hits,
+        block_commit(s_q.A.sums, s_q.A.hdr->W, T.sx, T.sx2, T.hits, T.checked, 0, s_err, s_x, s_x2lo, s_x2hi, s_hits,
                      s_checked);
-        T = ThreadSums();
+        T.clear();
         if (threadIdx.x == 0) {
           s_err = 0;
           s_x = s_x2lo = s_x2hi = s_hits = s_checked = 0;
         }
+        __syncthreads();  // the record is no longer read
       }
       if (q >= nq) break;
       // the records are kBatchQueryBytes apart
@@ -1505,50 +1777,78 @@ __global__ void __launch_bounds__(BS, (256 * TC_SAMPLE_MIN_BLOCKS) / BS)
       for (uint32_t w = threadIdx.x; w < sizeof(BatchQuery) / 16; w += BS) dst[w] = src[w];
       __syncthreads();
       cur = q;
-      bad = index_check(s_q.A, s_q.P);
-      W = s_q.A.hdr->W;
-      shift = s_q.A.hdr->shift;
-      if (bad && threadIdx.x == 0) atomicOr(&sums[q].err, bad);
+      const uint32_t e = index_check(s_q.A, s_q.P);
+      bad = e != 0;
+      if (bad && threadIdx.x == 0) atomicOr(&s_q.A.sums->err, e);
     }
+    const uint64_t W = s_q.A.hdr->W;
+    const uint32_t shift = s_q.A.hdr->shift;
     if (!bad && W) {
-      const uint64_t j0 = (item - tile_begin[q]) * tile;
-      const uint64_t j1 = j0 + tile < s_q.A.count ? j0 + tile : s_q.A.count;
-      const uint32_t* order = s_q.A.order;
-      for (uint64_t j = j0 + threadIdx.x; j < j1; j += BS) {
-        const uint64_t i = order ? (j & ~(kChunkSamples - 1)) + __ldg(order + j) : j;
-        sample_one<false>(s_q.A, s_q.P, W, shift, i, T, &s_err);
+      const uint64_t j = s_j, nb = s_q.A.ord.nb;
+      uint64_t j0 = j * tile, j1 = min(j0 + tile, s_q.A.count);
+      bool ordered = false;
+      if (nb) {  // as batch_record_group
+        const uint64_t gr = max((uint64_t)tile * nb / s_q.A.count, (uint64_t)1);
+        const uint64_t b0 = j * gr, b1 = min(b0 + gr, nb);
+        ordered = s_q.A.ord.head[0] == 0;
+        // (at most 2^28 samples and 2^20 buckets: the products fit)
+        j0 = ordered ? b0 : s_q.A.count * b0 / nb;
+        j1 = ordered ? b1 : s_q.A.count * b1 / nb;
+      }
+      if (ordered) {
+#pragma unroll 1
+        for (uint32_t b = (uint32_t)j0; b < (uint32_t)j1; b++)
+          sample_bucket<BS, false, Compact>(s_q.A, s_q.P, W, shift, b, S, T, nullptr, 0);
+      } else {
+        sample_ids<BS, false, Compact>(s_q.A, s_q.P, W, shift, j0 + threadIdx.x, j1, BS, T, nullptr, 0);
       }
     }
     __syncthreads();
   }
 }
 
-int sample_batch_blocks_per_sm(int bs) {
-  static int cache[3] = {0, 0, 0};
-  const int i = bs == 128 ? 0 : bs == 256 ? 1 : bs == 512 ? 2 : -1;
-  if (i < 0) return 0;
-  if (!cache[i]) {
+template <int BS, bool Compact>
+static int batch_blocks_per_sm() {
+  static int cached = 0;
+  if (!cached) {
     int b = 0;
-    if (bs == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample_batch<128>, 128, 0);
-    if (bs == 256) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample_batch<256>, 256, 0);
-    if (bs == 512) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample_batch<512>, 512, 0);
-    cache[i] = b > 0 ? b : 1;
+    cudaFuncSetAttribute(k_sample_batch<BS, Compact>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(TileShared<BS>));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample_batch<BS, Compact>, BS, sizeof(TileShared<BS>));
+    cached = b > 0 ? b : 1;
   }
-  return cache[i];
+  return cached;
 }
 
-tc_status launch_sample_batch(int bs, uint32_t tile, unsigned blocks, const void* d_records,
-                              const uint64_t* d_tile_begin, uint32_t nq, unsigned long long* d_next_item,
-                              SampleSums* d_sums, cudaStream_t st) {
-  const char* Q = (const char*)d_records;
-  if (bs == 128)
-    k_sample_batch<128><<<blocks, 128, 0, st>>>(Q, d_tile_begin, nq, tile, d_next_item, d_sums);
-  else if (bs == 256)
-    k_sample_batch<256><<<blocks, 256, 0, st>>>(Q, d_tile_begin, nq, tile, d_next_item, d_sums);
-  else if (bs == 512)
-    k_sample_batch<512><<<blocks, 512, 0, st>>>(Q, d_tile_begin, nq, tile, d_next_item, d_sums);
+int sample_batch_blocks_per_sm(int bs, bool compact) {
+  if (bs == 128) return compact ? batch_blocks_per_sm<128, true>() : batch_blocks_per_sm<128, false>();
+  if (bs == 256) return compact ? batch_blocks_per_sm<256, true>() : batch_blocks_per_sm<256, false>();
+  if (bs == 512) return compact ? batch_blocks_per_sm<512, true>() : batch_blocks_per_sm<512, false>();
+  return 0;
+}
+
+
+template <int BS>
+static void launch_batch(bool compact, uint32_t tile, unsigned blocks, const char* Q, const uint64_t* d_tile_begin,
+                         uint32_t nq, unsigned long long* d_next_item, cudaStream_t st) {
+  if (compact)
+    k_sample_batch<BS, true><<<blocks, BS, sizeof(TileShared<BS>), st>>>(Q, d_tile_begin, nq, tile, d_next_item);
   else
+    k_sample_batch<BS, false><<<blocks, BS, sizeof(TileShared<BS>), st>>>(Q, d_tile_begin, nq, tile, d_next_item);
+}
+
+tc_status launch_sample_batch(int bs, bool compact, uint32_t tile, unsigned blocks, const void* d_records,
+                              const uint64_t* d_tile_begin, uint32_t nq, unsigned long long* d_next_item,
+                              cudaStream_t st) {
+  const char* Q = (const char*)d_records;
+  if (!sample_batch_blocks_per_sm(bs, compact))
     return set_error(TC_ERR_INVALID_ARG, "batch block size must be 128, 256 or 512");
+  if (bs == 128)
+    launch_batch<128>(compact, tile, blocks, Q, d_tile_begin, nq, d_next_item, st);
+  else if (bs == 256)
+    launch_batch<256>(compact, tile, blocks, Q, d_tile_begin, nq, d_next_item, st);
+  else
+    launch_batch<512>(compact, tile, blocks, Q, d_tile_begin, nq, d_next_item, st);
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());
   return TC_OK;
