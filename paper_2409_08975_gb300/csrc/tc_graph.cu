@@ -640,11 +640,12 @@ __global__ void k_anchor_out(const OutEdge* __restrict__ out_e, const InEdge* __
 // Each pair is inserted once; a probe sequence ends at the first empty slot,
 // which exists because the load factor is at most 1/2.
 __global__ void k_pair_hash(const uint32_t* __restrict__ pair_src, const int32_t* __restrict__ pair_dst,
-                            const uint32_t* __restrict__ pair_eoff, uint32_t P, PairSlot* table, uint64_t mask) {
+                            const uint32_t* __restrict__ pair_eoff, uint32_t P, PairSlot* table, uint32_t mask,
+                            int shift) {
   for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t x = pair_src[p], y = (uint32_t)pair_dst[p];
     const unsigned long long key = pair_key(x, y);
-    uint64_t h = mix64(key) & mask;
+    uint32_t h = pair_slot(x, y, shift);
     for (uint64_t probe = 0; probe <= mask; probe++) {
       unsigned long long* word = reinterpret_cast<unsigned long long*>(&table[h]);
       if (atomicCAS(word, kEmptyPairKey, key) == kEmptyPairKey) {
@@ -859,12 +860,18 @@ tc_status build_graph(int64_t n, int64_t m, const int32_t* d_src, const int32_t*
   TRY_C(cudaGetLastError(), "k_offsets");
   // pair hash table, capacity the power of two >= max(2, 2P)
   uint64_t cap = 2;
-  while (cap < 2ull * P) cap <<= 1;
-  g->hash_mask = cap - 1;
+  g->hash_shift = 63;
+  while (cap < 2ull * P) {
+    cap <<= 1;
+    g->hash_shift--;
+  }
+  if (cap > 1ull << 32) return done(set_error(TC_ERR_OOM, "pair table larger than the device's memory"));
+  g->hash_mask = (uint32_t)(cap - 1);
   TRY_S(dmalloc(&g->pair_hash, cap, st));
   TRY_C(cudaMemsetAsync(g->pair_hash, 0xFF, sizeof(PairSlot) * cap, st), "memset");
   if (P) {
-    k_pair_hash<<<grid_for(P), 256, 0, st>>>(pair_src, g->pair_dst, g->pair_eoff, P, g->pair_hash, g->hash_mask);
+    k_pair_hash<<<grid_for(P), 256, 0, st>>>(pair_src, g->pair_dst, g->pair_eoff, P, g->pair_hash, g->hash_mask,
+                                             g->hash_shift);
     TC_LAUNCHED(1);
     TRY_C(cudaGetLastError(), "k_pair_hash");
   }

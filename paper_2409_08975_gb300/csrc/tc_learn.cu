@@ -58,11 +58,10 @@ __device__ __forceinline__ uint32_t count_window(const OutEdge* __restrict__ out
   return search_time<false>(a, b, hi, tt) - search_time<true>(a, b, lo, tt);
 }
 
-__device__ __forceinline__ uint32_t pair_count(const PairSlot* __restrict__ table, uint64_t mask,
+__device__ __forceinline__ uint32_t pair_count(const PairSlot* __restrict__ table, uint32_t mask, int shift,
                                                const int64_t* __restrict__ pair_t, int32_t x, int32_t y, int64_t lo,
                                                int64_t hi) {
-  const uint64_t key = pair_key((uint32_t)x, (uint32_t)y);
-  uint64_t h = mix64(key) & mask;
+  uint32_t h = pair_slot((uint32_t)x, (uint32_t)y, shift);
   for (uint64_t probe = 0; probe <= mask; probe++) {
     const uint4 slot = __ldg(reinterpret_cast<const uint4*>(table + h));
     if (slot.x == (uint32_t)x && slot.y == (uint32_t)y) {
@@ -79,7 +78,7 @@ __device__ __forceinline__ uint32_t pair_count(const PairSlot* __restrict__ tabl
 __global__ void __launch_bounds__(256) k_features(const OutEdge* __restrict__ out_e,
                                                   const uint32_t* __restrict__ out_off,
                                                   const InEdge* __restrict__ in_e, const uint32_t* __restrict__ in_off,
-                                                  const PairSlot* __restrict__ table, uint64_t mask,
+                                                  const PairSlot* __restrict__ table, uint32_t mask, int shift,
                                                   const int64_t* __restrict__ pair_t, const EdgeWin* __restrict__ win,
                                                   uint64_t m, int64_t delta, __nv_bfloat16* __restrict__ feat) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -100,8 +99,8 @@ __global__ void __launch_bounds__(256) k_features(const OutEdge* __restrict__ ou
     c[4] = (float)count_window(out_e, out_off, in_e, in_off, false, e.src, lo, hi);
     c[5] = (float)count_window(out_e, out_off, in_e, in_off, true, e.dst, lo, hi);
     c[6] = (float)count_window(out_e, out_off, in_e, in_off, false, e.dst, lo, hi);
-    c[7] = (float)pair_count(table, mask, pair_t, e.src, e.dst, lo, hi);
-    c[8] = (float)pair_count(table, mask, pair_t, e.dst, e.src, lo, hi);
+    c[7] = (float)pair_count(table, mask, shift, pair_t, e.src, e.dst, lo, hi);
+    c[8] = (float)pair_count(table, mask, shift, pair_t, e.dst, e.src, lo, hi);
     c[9] = (float)(__ldg(out_off + e.src + 1) - __ldg(out_off + e.src));
     c[10] = (float)(__ldg(in_off + e.dst + 1) - __ldg(in_off + e.dst));
     c[11] = (float)(__ldg(in_off + e.src + 1) - __ldg(in_off + e.src));
@@ -1375,7 +1374,7 @@ tc_status launch_features(const tc_graph* g, const EdgeWin* win, int64_t delta, 
   const uint64_t m = (uint64_t)g->m;
   if (!m) return TC_OK;
   k_features<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(g->out_e, g->out_off, g->in_e, g->in_off, g->pair_hash,
-                                                          g->hash_mask, g->pair_t, win, m, delta,
+                                                          g->hash_mask, g->hash_shift, g->pair_t, win, m, delta,
                                                           reinterpret_cast<__nv_bfloat16*>(feat));
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());

@@ -489,7 +489,8 @@ struct SamplerArgs {
   const OutEdge* out_e;
   const InEdge* in_e;
   const PairSlot* pair_hash;
-  uint64_t hash_mask;
+  uint32_t hash_mask;
+  int hash_shift;
   const int64_t* pair_t;
   const uint32_t* pair_t32;  // pair-list times as t - tmin, or NULL
   int64_t tmin;
@@ -549,7 +550,7 @@ struct SampleTime<false> {
 // y) from the pair hash table, one 16-byte slot per probe.
 __device__ __forceinline__ void pair_list(const SamplerArgs& A, int32_t x, int32_t y, uint32_t* s, uint32_t* e) {
   *s = *e = 0;
-  uint64_t h = mix64(pair_key((uint32_t)x, (uint32_t)y)) & A.hash_mask;
+  uint32_t h = pair_slot((uint32_t)x, (uint32_t)y, A.hash_shift);
   for (uint64_t probe = 0; probe <= A.hash_mask; probe++) {
     const uint4 slot = __ldg(reinterpret_cast<const uint4*>(A.pair_hash + h));
     if (slot.x == (uint32_t)x && slot.y == (uint32_t)y) {
@@ -563,14 +564,21 @@ __device__ __forceinline__ void pair_list(const SamplerArgs& A, int32_t x, int32
 }
 
 // Positions [*a, *b) of the non-empty pair list [s, e) with time in (tlo,
-// thi]: the first positions with time > tlo and with time > thi.  Both
-// bisections halve the same length, so one loop runs them with a probe of
-// each in flight.
+// thi]: the first positions with time > tlo and with time > thi.  Nine in ten
+// lists that are found have no entry in the window, most because they end
+// before it or begin after it, which their two ends tell at once; both
+// bisections of the others halve the same length, so one loop runs them with
+// a probe of each in flight.
 template <bool Compact>
 __device__ __forceinline__ void pair_window(const SamplerArgs& A, uint32_t s, uint32_t e,
                                             typename SampleTime<Compact>::T tlo, typename SampleTime<Compact>::T thi,
                                             uint32_t* a, uint32_t* b) {
   typedef SampleTime<Compact> Tm;
+  const typename Tm::T first = Tm::pair(A, s), last = Tm::pair(A, e - 1);
+  if (last <= tlo || first > thi) {
+    *a = *b = s;
+    return;
+  }
   uint32_t pa = s, pb = s;
   for (uint32_t len = e - s; len > 1;) {
     const uint32_t half = len >> 1;
@@ -841,11 +849,22 @@ __device__ __forceinline__ void block_commit(SampleSums* G, uint64_t W, uint64_t
 // Exhaustive path sum (the proof of Claim 2): path p in [0, W) is the
 // (p - prefix[e])-th pair (p1, p3) of middle edge e, p1 major; the sum of
 // CheckMotif over all paths is the exact count C, the sum of squares gives
-// the exact variance of one sample.  Paths [first, first + count).
+// the exact variance of one sample.
+//
+// A warp takes runs of kPathRun consecutive paths, lane l every 32nd of them
+// from l on: the middle edge and its windows, and the end edge e1, are loaded
+// when a lane crosses into the next one (an edge has thousands of paths where
+// an exact count takes long), and the pair (p1, p3) is stepped on, so that a
+// path costs one coalesced end-edge load and its pair lookup.  Bound by issue
+// (62% of the slots, 97% of the loads hit L1); 4.0e9 paths of a 3e6-edge
+// graph: 26.2 ms (41.2 ms with a CDF search, a 64-bit division and both end
+// loads per path; 28.5 ms without pair_window's look at the list's ends).
+// Four blocks of 256 (64 registers): with five 29.9 ms, with six 33.9 ms.
+constexpr uint64_t kPathRun = 4096;
 template <bool Compact>
 __global__ void __launch_bounds__(256, 4) k_path_sum(const __grid_constant__ SamplerArgs A,
-                                                                            const __grid_constant__ Plan P,
-                                                                            uint64_t first, uint64_t count) {
+                                                    const __grid_constant__ Plan P) {
+  typedef SampleTime<Compact> Tm;
   const IndexHeader* H = A.hdr;
   const uint64_t W = H->W;
   const uint32_t shift = H->shift;
@@ -862,31 +881,71 @@ __global__ void __launch_bounds__(256, 4) k_path_sum(const __grid_constant__ Sam
     return;
   }
   ThreadSums T(&s_err);
-  const uint64_t end = first + count < W ? first + count : W;
-  for (uint64_t p = first + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < end;
-       p += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t b = (uint32_t)(p >> shift);
-    uint32_t lo = __ldg(A.guide + b), hi = __ldg(A.guide + b + 1);
-    while (lo < hi) {
-      const uint32_t mid = lo + ((hi - lo + 1) >> 1);
-      if (__ldg(A.prefix + mid) <= p) lo = mid; else hi = mid - 1;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  uint64_t hits = 0, checked = 0;  // a thread may take more than 2^32 paths
+  for (uint64_t run = warp * kPathRun; run < W; run += warps * kPathRun) {
+    const uint64_t end = W - run < kPathRun ? W : run + kPathRun;
+    uint64_t stop = 0;  // end of the paths of the current middle edge
+    uint32_t lo1 = 0, lo3 = 0, d3 = 1, i1 = 0, i3 = 0;
+    int32_t u = 0, v = 0, up = 0, vp = 0;
+    typename Tm::T t1 = 0, t2 = 0, t3 = 0;
+#pragma unroll 1
+    for (uint64_t p = run + (threadIdx.x & 31); p < end; p += 32) {
+      if (p >= stop) {
+        const uint32_t b = (uint32_t)(p >> shift);
+        uint32_t lo = __ldg(A.guide + b), hi = __ldg(A.guide + b + 1);
+        while (lo < hi) {
+          const uint32_t mid = lo + ((hi - lo + 1) >> 1);
+          if (__ldg(A.prefix + mid) <= p) lo = mid; else hi = mid - 1;
+        }
+        if (lo >= A.m) { T.fail(kErrBounds); continue; }
+        const EdgeWin wn = A.win[lo];
+        const OutEdge e = A.out_e[lo];
+        if (wn.d1 == 0 || wn.d3 == 0) { T.fail(kErrBounds); continue; }
+        u = e.src;
+        v = e.dst;
+        t2 = Tm::rel(A, e.t);
+        lo1 = wn.lo1;
+        lo3 = wn.lo3;
+        d3 = wn.d3;
+        const uint64_t first = __ldg(A.prefix + lo), j = p - first;
+        stop = __ldg(A.prefix + lo + 1);
+        if (j >> 32) {
+          i1 = (uint32_t)(j / d3);
+          i3 = (uint32_t)(j % d3);
+        } else {
+          i1 = (uint32_t)j / d3;
+          i3 = (uint32_t)j - i1 * d3;
+        }
+        if (lo1 + i1 >= A.m || (uint64_t)lo3 + d3 > A.m) {
+          T.fail(kErrBounds);
+          stop = 0;
+          continue;
+        }
+        end_edge<Compact>(A, P.alpha1, lo1 + i1, &up, &t1);
+      } else {
+        i3 += 32;
+        if (i3 >= d3) {
+          const uint32_t q = i3 / d3;
+          i1 += q;
+          i3 -= q * d3;
+          if (lo1 + i1 >= A.m) {
+            T.fail(kErrBounds);
+            stop = 0;
+            continue;
+          }
+          end_edge<Compact>(A, P.alpha1, lo1 + i1, &up, &t1);
+        }
+      }
+      end_edge<Compact>(A, P.alpha3, lo3 + i3, &vp, &t3);
+      T.add(check_motif<Compact>(A, P, up, u, v, vp, t1, t2, t3, &s_err, &T.checked));
     }
-    if (lo >= A.m) { T.fail(kErrBounds); continue; }
-    const EdgeWin wn = A.win[lo];
-    const OutEdge e = A.out_e[lo];
-    if (wn.d1 == 0 || wn.d3 == 0) { T.fail(kErrBounds); continue; }
-    const uint64_t j = p - __ldg(A.prefix + lo);
-    const uint32_t p1 = wn.lo1 + (uint32_t)(j / wn.d3), p3 = wn.lo3 + (uint32_t)(j % wn.d3);
-    if (p1 >= A.m || p3 >= A.m) { T.fail(kErrBounds); continue; }
-    int32_t up, vp;
-    typename SampleTime<Compact>::T t1, t3;
-    end_edge<Compact>(A, P.alpha1, p1, &up, &t1);
-    end_edge<Compact>(A, P.alpha3, p3, &vp, &t3);
-    const uint64_t X = check_motif<Compact>(A, P, up, e.src, e.dst, vp, t1, SampleTime<Compact>::rel(A, e.t), t3,
-                                            &s_err, &T.checked);
-    T.add(X);
+    hits += T.hits;
+    checked += T.checked;
+    T.hits = T.checked = 0;
   }
-  block_commit(A.sums, W, T.sx, T.sx2, T.hits, T.checked, 0, s_err, s_x, s_x2lo, s_x2hi, s_hits, s_checked);
+  block_commit(A.sums, W, T.sx, T.sx2, hits, checked, 0, s_err, s_x, s_x2lo, s_x2hi, s_hits, s_checked);
 }
 
 // The rejection loops: the first attempt is tested in the sampler itself and
@@ -1546,6 +1605,7 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
   A.in_e = g->in_e;
   A.pair_hash = g->pair_hash;
   A.hash_mask = g->hash_mask;
+  A.hash_shift = g->hash_shift;
   A.pair_t = g->pair_t;
   A.pair_t32 = TC_COMPACT_PAIRS ? g->pair_t32 : nullptr;
   A.tmin = g->tmin;
@@ -1637,6 +1697,7 @@ tc_status launch_path_sum(const tc_graph* g, const Plan& plan, int64_t delta, co
   A.in_e = g->in_e;
   A.pair_hash = g->pair_hash;
   A.hash_mask = g->hash_mask;
+  A.hash_shift = g->hash_shift;
   A.pair_t = g->pair_t;
   A.pair_t32 = TC_COMPACT_PAIRS ? g->pair_t32 : nullptr;
   A.tmin = g->tmin;
@@ -1654,7 +1715,7 @@ tc_status launch_path_sum(const tc_graph* g, const Plan& plan, int64_t delta, co
   uint64_t blocks = (uint64_t)num_sms() * (bps > 0 ? bps : 1);
   const uint64_t need = (W + 255) / 256;
   if (need < blocks) blocks = need ? need : 1;
-  kernel<<<(unsigned)blocks, 256, 0, st>>>(A, plan, 0, W);
+  kernel<<<(unsigned)blocks, 256, 0, st>>>(A, plan);
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());
   return TC_OK;
@@ -1687,6 +1748,7 @@ void batch_query_record(void* h_rec, const tc_graph* g, const Plan& plan, int64_
   A.in_e = g->in_e;
   A.pair_hash = g->pair_hash;
   A.hash_mask = g->hash_mask;
+  A.hash_shift = g->hash_shift;
   A.pair_t = g->pair_t;
   A.pair_t32 = TC_COMPACT_PAIRS ? g->pair_t32 : nullptr;
   A.tmin = g->tmin;

@@ -109,3 +109,24 @@ def test_buckets_that_outgrow_their_room(tc, tmp_path):
     subprocess.run([_build.nvcc()] + _build.ARCH + ["-shared", "-o", lib, obj] + rest + ["-cudart", "static"], check=True)
     r = subprocess.run([sys.executable, "-c", CHILD % (ROOT, os.path.join(ROOT, "tests")), lib], capture_output=True, text=True)
     assert r.returncode == 0 and "same sums" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("n,m,scale", [(6, 40, 1), (24, 900, 1), (24, 900, 1 << 33), (40, 5000, 1)])
+def test_path_sum_steps_over_small_windows(tc, n, m, scale):
+    # windows shorter than a warp's step, edges with fewer than 32 paths, and
+    # runs that end inside an edge, against the oracle's path sum
+    import torch
+    import oracle
+    from _graphs import small_random_graph
+    s, d, t = small_random_graph(m, n, m, 10 * m, dup_frac=0.3)
+    t = t * scale
+    dev = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=dt)  # noqa: E731
+    g = tc.tc_build_temporal_csr(n, dev(s, torch.int32), dev(d, torch.int32), dev(t, torch.int64))
+    og = oracle.build_csr(n, s, d, t)
+    for edges in (C4, CHORD, MULTI, TRIANGLE):
+        for delta in (20 * scale, 700 * scale):
+            plan = oracle.compile_motif(edges)
+            w = tc.tc_path_weights(g, tc.make_motif(edges), delta)
+            e = tc.tc_exact_count(g, tc.make_motif(edges), delta, w)
+            exp = oracle.path_sum(og, plan, delta)
+            assert (e["sum_x"], e["sum_x2"], e["W"]) == (exp["C"], exp["sum_x2"], exp["paths"]), (edges, delta)
