@@ -290,6 +290,50 @@ __device__ __forceinline__ uint32_t search_time(uint32_t lo, uint32_t hi, int64_
   return lo;
 }
 
+// First position p in [s, f) whose time is >= x (Gt: > x), searched from a
+// position a in [s, f]: doubling steps away from a until the answer is
+// bracketed, then bisection.  At most 2 log2(f - s) + 2 probes.
+template <bool Gt, class T, class TimeAt>
+__device__ __forceinline__ uint32_t gallop(uint32_t s, uint32_t f, uint32_t a, T x, TimeAt tt) {
+  auto pred = [&](uint32_t p) {
+    const T v = tt(p);
+    return Gt ? v > x : v >= x;
+  };
+  uint32_t lo, hi;  // the answer lies in [lo, hi]; pred(hi) holds or hi == f
+  if (a < f && !pred(a)) {
+    lo = a + 1;
+    hi = f;
+    uint32_t step = 1;
+    while (lo < hi) {
+      const uint32_t p = (hi - lo > step - 1) ? lo + (step - 1) : hi - 1;
+      if (pred(p)) {
+        hi = p;
+        break;
+      }
+      lo = p + 1;
+      step <<= 1;
+    }
+  } else {
+    lo = s;
+    hi = a;
+    uint32_t step = 1;
+    while (hi > lo) {
+      const uint32_t p = (hi - lo > step) ? hi - step : lo;
+      if (!pred(p)) {
+        lo = p + 1;
+        break;
+      }
+      hi = p;
+      step <<= 1;
+    }
+  }
+  while (lo < hi) {
+    const uint32_t mid = lo + ((hi - lo) >> 1);
+    if (pred(mid)) hi = mid; else lo = mid + 1;
+  }
+  return lo;
+}
+
 // Window of x's list (alpha < 0: in-list, else out-list) around time t
 // (beta < 0: before, else after; strict or closed at t) as positions [lo, hi).
 // The two bounds are searched independently so that their loads overlap.

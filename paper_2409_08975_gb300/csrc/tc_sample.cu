@@ -56,50 +56,6 @@ constexpr int kWThreads = 256;
 constexpr int kWItems = 8;
 constexpr int kWTile = kWThreads * kWItems;  // edges per tile: the scan's tile
 
-// First position p in [s, f) whose time is >= x (Gt: > x), searched from a
-// position a in [s, f]: doubling steps away from a until the answer is
-// bracketed, then bisection.  At most 2 log2(f - s) + 2 probes.
-template <bool Gt, class TimeAt>
-__device__ __forceinline__ uint32_t gallop(uint32_t s, uint32_t f, uint32_t a, int64_t x, TimeAt tt) {
-  auto pred = [&](uint32_t p) {
-    const int64_t v = tt(p);
-    return Gt ? v > x : v >= x;
-  };
-  uint32_t lo, hi;  // the answer lies in [lo, hi]; pred(hi) holds or hi == f
-  if (a < f && !pred(a)) {
-    lo = a + 1;
-    hi = f;
-    uint32_t step = 1;
-    while (lo < hi) {
-      const uint32_t p = (hi - lo > step - 1) ? lo + (step - 1) : hi - 1;
-      if (pred(p)) {
-        hi = p;
-        break;
-      }
-      lo = p + 1;
-      step <<= 1;
-    }
-  } else {
-    lo = s;
-    hi = a;
-    uint32_t step = 1;
-    while (hi > lo) {
-      const uint32_t p = (hi - lo > step) ? hi - step : lo;
-      if (!pred(p)) {
-        lo = p + 1;
-        break;
-      }
-      hi = p;
-      step <<= 1;
-    }
-  }
-  while (lo < hi) {
-    const uint32_t mid = lo + ((hi - lo) >> 1);
-    if (pred(mid)) hi = mid; else lo = mid + 1;
-  }
-  return lo;
-}
-
 // The window of list [s, f) around time t (beta < 0: before, else after;
 // strict or closed at t) as positions [*lo, *hi), searched from an anchor a
 // with lower_bound(t) <= a <= upper_bound(t).
@@ -107,11 +63,11 @@ template <class TimeAt>
 __device__ __forceinline__ void window_from(uint32_t s, uint32_t f, uint32_t a, int beta, int closed, int64_t t,
                                             int64_t delta, TimeAt tt, uint32_t* lo, uint32_t* hi) {
   if (beta < 0) {
-    *hi = closed ? gallop<true>(s, f, a, t, tt) : gallop<false>(s, f, a, t, tt);
-    *lo = gallop<false>(s, f, *hi, sat_sub(t, delta), tt);
+    *hi = closed ? gallop<true, int64_t>(s, f, a, t, tt) : gallop<false, int64_t>(s, f, a, t, tt);
+    *lo = gallop<false, int64_t>(s, f, *hi, sat_sub(t, delta), tt);
   } else {
-    *lo = closed ? gallop<false>(s, f, a, t, tt) : gallop<true>(s, f, a, t, tt);
-    *hi = gallop<true>(s, f, *lo, sat_add(t, delta), tt);
+    *lo = closed ? gallop<false, int64_t>(s, f, a, t, tt) : gallop<true, int64_t>(s, f, a, t, tt);
+    *hi = gallop<true, int64_t>(s, f, *lo, sat_add(t, delta), tt);
   }
 }
 
@@ -230,11 +186,11 @@ __device__ __forceinline__ void side_window_rw(const WeightsArgs& A, int alpha, 
   const uint32_t* t32 = alpha < 0 ? A.in_t32 : A.out_t32;
   auto tt = [&](uint32_t p) -> int64_t { return (int64_t)__ldg(t32 + p) + A.tmin; };
   if (beta < 0) {
-    *hi = (exact && !A.closed) ? a : (A.closed ? gallop<true>(s, f, a, t, tt) : gallop<false>(s, f, a, t, tt));
-    *lo = gallop<false>(s, f, *hi, sat_sub(t, A.delta), tt);
+    *hi = (exact && !A.closed) ? a : (A.closed ? gallop<true, int64_t>(s, f, a, t, tt) : gallop<false, int64_t>(s, f, a, t, tt));
+    *lo = gallop<false, int64_t>(s, f, *hi, sat_sub(t, A.delta), tt);
   } else {
-    *lo = (exact && A.closed) ? a : (A.closed ? gallop<false>(s, f, a, t, tt) : gallop<true>(s, f, a, t, tt));
-    *hi = gallop<true>(s, f, *lo, sat_add(t, A.delta), tt);
+    *lo = (exact && A.closed) ? a : (A.closed ? gallop<false, int64_t>(s, f, a, t, tt) : gallop<true, int64_t>(s, f, a, t, tt));
+    *hi = gallop<true, int64_t>(s, f, *lo, sat_add(t, A.delta), tt);
   }
 }
 

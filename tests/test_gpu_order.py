@@ -130,3 +130,30 @@ def test_path_sum_steps_over_small_windows(tc, n, m, scale):
             e = tc.tc_exact_count(g, tc.make_motif(edges), delta, w)
             exp = oracle.path_sum(og, plan, delta)
             assert (e["sum_x"], e["sum_x2"], e["W"]) == (exp["C"], exp["sum_x2"], exp["paths"]), (edges, delta)
+
+
+@pytest.mark.parametrize("name,m,delta", [("bursty", 60_000, 0), ("bursty", 60_000, 3600), ("bursty", 2047, 86_400),
+                                          ("bursty", 2049, 1 << 40), ("hub", 400_000, 3000), ("hub", 400_000, 0)])
+def test_features_of_32_and_64_bit_times_are_the_same(tc, name, m, delta):
+    # the same graph in units a thousand times finer has times beyond 32 bits
+    # and takes the other kernel; the counts, so the rows, are the same bits
+    import torch
+    from paper_2409_08975_gb300 import synth
+    if name == "hub":  # lists of 200,000 entries on two vertices: saturated range words
+        rng = np.random.default_rng(3)
+        other = rng.integers(2, 5000, m)
+        src, dst = np.where(rng.random(m) < 0.5, 0, other), np.where(rng.random(m) < 0.5, 1, rng.integers(2, 5000, m))
+        keep = src != dst
+        c = {"n": 5000, "src": src[keep], "dst": dst[keep], "t": rng.integers(0, 10_000_000, m)[keep]}
+    else:
+        c = synth.scaled_mid(max(100, m // 20), m, seed=m)
+    dev = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=dt)  # noqa: E731
+    rows = []
+    for scale in (1, 1000):
+        g = tc.tc_build_temporal_csr(c["n"], dev(c["src"], torch.int32), dev(c["dst"], torch.int32),
+                                     dev(c["t"].astype(np.int64) * scale, torch.int64))
+        assert (g.t_max - g.t_min < 1 << 32) == (scale == 1)
+        w = tc.tc_path_weights(g, tc.make_motif(CHORD, window=1), delta * scale)
+        assert w.W > 0 or delta == 0
+        rows.append(tc.tc_edge_features(g, tc.make_motif(CHORD, window=1), delta * scale, w).view(torch.int16))
+    assert torch.equal(rows[0], rows[1])
