@@ -693,20 +693,21 @@ tc_status tc_mlp_grad_ex(const tc_mlp* mlp, const uint16_t* d_feat, const uint32
   if (objective == TC_OBJECTIVE_VARIANCE && !(eps > 0.f)) return set_error(TC_ERR_INVALID_ARG, "eps must be > 0");
   const bool var = objective == TC_OBJECTIVE_VARIANCE, bce = objective == TC_OBJECTIVE_BCE;
   cudaStream_t st = S(stream);
-  // loss, spare float, then (variance) logits and dloss/dz or (BCE) the clipped labels
+  // loss, then from the 256th byte on the variance objective's scratch or (BCE) the clipped labels
   float* buf = nullptr;
-  TC_CUDA(pool_malloc(&buf, sizeof(float) * (2 + (var ? 2 * (n ? n : 1) : (bce ? (n ? n : 1) : 0))), st));
+  TC_CUDA(pool_malloc(&buf, 256 + (var ? variance_scratch_bytes(n) : sizeof(float) * (bce ? n : 0)), st));
+  float* rest = buf + 64;
   float* loss = buf;
   tc_status s = TC_OK;
   cudaError_t e = cudaMemsetAsync(d_grad, 0, sizeof(float) * TC_MLP_PARAMS, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(buf, 0, sizeof(float) * 2, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(buf, 0, sizeof(float), st);
   if (e != cudaSuccess) s = cuda_status(e, "memset");
   if (s == TC_OK) {
     if (var) {
-      s = launch_variance_grad(mlp, d_feat, d_rows, d_labels, n, eps, d_grad, loss, buf + 2, buf + 2 + n, buf + 1, st);
+      s = launch_variance_grad(mlp, d_feat, d_rows, d_labels, n, eps, d_grad, loss, rest, st);
     } else if (bce) {
-      s = launch_clip_labels(d_labels, n, buf + 2, st);
-      if (s == TC_OK) s = launch_mlp_grad(mlp, d_feat, d_rows, buf + 2, n, d_grad, loss, st);
+      s = launch_clip_labels(d_labels, n, rest, st);
+      if (s == TC_OK) s = launch_mlp_grad(mlp, d_feat, d_rows, rest, n, d_grad, loss, st);
     } else {
       s = launch_mlp_grad(mlp, d_feat, d_rows, d_labels, n, d_grad, loss, st);
     }
@@ -750,13 +751,13 @@ tc_status tc_mlp_train_ex(tc_mlp* mlp, const tc_graph* g, const tc_motif* motif,
   uint32_t* rows = nullptr;
   float* labels = nullptr;
   float* losses = nullptr;
-  float* zbuf = nullptr;  // variance objective: logits, dloss/dz and a spare float of a batch
+  void* vbuf = nullptr;  // variance objective: scratch of a batch
   SampleSums* sums = nullptr;
   tc_status s = TC_OK;
   const bool var = objective == TC_OBJECTIVE_VARIANCE;
   const uint64_t bmax = batch < n_samples ? batch : n_samples;
   cudaError_t e = pool_malloc(&trace, 32 * n_samples, st);
-  if (e == cudaSuccess && var) e = pool_malloc(&zbuf, sizeof(float) * (2 * bmax + 1), st);
+  if (e == cudaSuccess && var) e = pool_malloc(&vbuf, variance_scratch_bytes(bmax), st);
   if (e == cudaSuccess) e = pool_malloc(&rows, 4 * n_samples, st);
   if (e == cudaSuccess) e = pool_malloc(&labels, 4 * n_samples, st);
   if (e == cudaSuccess) e = pool_malloc(&losses, sizeof(float) * steps, st);
@@ -770,8 +771,8 @@ tc_status tc_mlp_train_ex(tc_mlp* mlp, const tc_graph* g, const tc_motif* motif,
   for (uint64_t b = 0; b < steps && s == TC_OK; b++) {
     const uint64_t lo = b * batch, nb = (n_samples - lo) < batch ? (n_samples - lo) : batch;
     if (var)
-      s = launch_variance_grad(mlp, d_feat, rows + lo, labels + lo, nb, eps, mlp_grad_buffer(mlp), losses + b, zbuf,
-                               zbuf + bmax, zbuf + 2 * bmax, st);
+      s = launch_variance_grad(mlp, d_feat, rows + lo, labels + lo, nb, eps, mlp_grad_buffer(mlp), losses + b, vbuf,
+                               st);
     else
       s = launch_mlp_grad(mlp, d_feat, rows + lo, labels + lo, nb, mlp_grad_buffer(mlp), losses + b, st);
     if (s == TC_OK) s = mlp_adam(mlp, lr, st);
@@ -785,7 +786,7 @@ tc_status tc_mlp_train_ex(tc_mlp* mlp, const tc_graph* g, const tc_motif* motif,
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_mlp_train");
   }
-  for (void* p : {(void*)trace, (void*)rows, (void*)labels, (void*)losses, (void*)sums, (void*)zbuf})
+  for (void* p : {(void*)trace, (void*)rows, (void*)labels, (void*)losses, (void*)sums, vbuf})
     if (p) cudaFreeAsync(p, st);
   if (s == TC_OK && hs.err) s = device_status(hs.err, "tc_mlp_train");
   if (s == TC_OK && var) s = mlp_check_error(mlp, st, "tc_mlp_train");

@@ -1112,23 +1112,16 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
 
 // ---------------------------------------------------------------------------
 // Gradient of the mean closure loss over a batch (the binary cross-entropy
-// when every label is 0 or 1), or of any loss whose dloss/dz3 per row is
-// given.  Each warp runs the forward of a 16-row tile on the tensor cores and
+// when every label is 0 or 1), or (V given) of the estimator-variance
+// objective.  Each warp runs the forward of a 16-row tile on the tensor cores and
 // back-propagates in FP32:
-//   dz3 = (-y (1 - g) if y > 0 else g) / B with g = sigmoid(z3) (or the given
-//   dz3), dz2 = dz3 W3 * [z2 > 0], dz1 = W2^T dz2 * [z1 > 0];
+//   dz3 = (-y (1 - g) if y > 0 else g) / B with g = sigmoid(z3) (or the
+//   variance objective's), dz2 = dz3 W3 * [z2 > 0], dz1 = W2^T dz2 * [z1 > 0];
 // the per-row vectors go to shared memory, where the block accumulates the
 // parameter gradients (each thread owns a fixed set of parameters) before one
 // global atomic add per parameter and block.
 
 constexpr int kTrainWarps = 4;
-// Row tiles of kTrainRows per block of the gradient launch: one tile per
-// block puts four times more blocks in flight than four tiles (the parameter
-// gradients then take more global atomics, which cost less than the idle
-// SMs did: 48 ms instead of 111 ms for 1e7 training rows on the 20M-edge graph).
-#ifndef TC_TRAIN_TILES
-#define TC_TRAIN_TILES 1
-#endif
 constexpr int kTrainRows = 16 * kTrainWarps;
 
 // Row strides of the backward's per-row arrays (FP32), padded so that the
@@ -1169,24 +1162,39 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1
 // Estimator-variance objective over a batch of n rows: with h_i = eps + g_i,
 // g_i = sigmoid(z_i), the per-sample second moment of the estimate under the
 // proposal is proportional to L = mean(h) * mean(X_i^2 / h_i) (the batch's
-// paths come from the plain sampler, so mean(h) estimates Q / W).  Writes
-// dL/dz_i into dz and L into *loss.  The per-row terms are FP32 (the
-// objective is checked to 1e-3 and its gradient to 1e-2; FP64 arithmetic
-// runs at a small fraction of the FP32 rate on this GPU, and a division per
-// row in FP64 made this kernel the bulk of a training step); only the sums
-// over the batch accumulate in FP64.
-__global__ void __launch_bounds__(1024) k_variance_dz(const float* __restrict__ z, const float* __restrict__ X,
-                                                      uint64_t n, float eps, float* __restrict__ dz,
-                                                      float* __restrict__ loss) {
-  __shared__ double s_a[32], s_b[32];
-  __shared__ double s_A, s_B;
+// paths come from the plain sampler, so mean(h) estimates Q / W).  Forms
+// A = mean(h), B = mean(X^2 / h) and L in *loss; the gradient kernel takes
+// dL/dz_i from them row by row.  The per-row terms are FP32 (the objective is
+// checked to 1e-3 and its gradient to 1e-2; FP64 arithmetic runs at a small
+// fraction of the FP32 rate on this GPU, and a division per row in FP64 made
+// this kernel the bulk of a training step); only the sums over the batch
+// accumulate in FP64.  Blocks of 1024 rows add their sums, the last to finish
+// forms the means: 7 us for 16,384 rows, 31 us in one block that also wrote
+// dL/dz for every row.
+struct VarianceSums {  // zero before each launch; A, B are its results
+  double h, x2;
+  unsigned int done;
+  float A, B;
+};
+constexpr int kVarThreads = 256;
+constexpr int kVarRows = 1024;
+
+__global__ void __launch_bounds__(kVarThreads) k_variance_sums(const float* __restrict__ z,
+                                                              const float* __restrict__ X, uint64_t n, float eps,
+                                                              VarianceSums* __restrict__ V, float* __restrict__ loss) {
+  __shared__ double s_a[kVarThreads / 32], s_b[kVarThreads / 32];
   double a = 0.0, b = 0.0;
-  for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const float h = eps + sigmoidf_(z[i]);
-    const float x = X[i];
-    a += (double)h;
-    b += (double)(x * x / h);
+#pragma unroll
+  for (int it = 0; it < kVarRows / kVarThreads; it++) {
+    const uint64_t i = (uint64_t)blockIdx.x * kVarRows + (uint64_t)it * kVarThreads + threadIdx.x;
+    if (i < n) {
+      const float h = eps + sigmoidf_(z[i]);
+      const float x = X[i];
+      a += (double)h;
+      b += (double)(x * x / h);
+    }
   }
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
@@ -1198,21 +1206,19 @@ __global__ void __launch_bounds__(1024) k_variance_dz(const float* __restrict__ 
   __syncthreads();
   if (threadIdx.x == 0) {
     double ta = 0.0, tb = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
+    for (int w = 0; w < kVarThreads / 32; w++) {
       ta += s_a[w];
       tb += s_b[w];
     }
-    s_A = ta / (double)n;
-    s_B = tb / (double)n;
-    *loss = (float)(s_A * s_B);
-  }
-  __syncthreads();
-  const float A = (float)s_A, B = (float)s_B, inv_n = (float)(1.0 / (double)n);
-  for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const float g = sigmoidf_(z[i]);
-    const float h = eps + g;
-    const float x = X[i];
-    dz[i] = g * (1.f - g) * (B - A * (x / h) * (x / h)) * inv_n;
+    atomicAdd(&V->h, ta);
+    atomicAdd(&V->x2, tb);
+    __threadfence();
+    if (atomicAdd(&V->done, 1u) == gridDim.x - 1) {
+      const double A = atomicAdd(&V->h, 0.0) / (double)n, B = atomicAdd(&V->x2, 0.0) / (double)n;
+      V->A = (float)A;
+      V->B = (float)B;
+      *loss = (float)(A * B);
+    }
   }
 }
 
@@ -1221,7 +1227,9 @@ __global__ void __launch_bounds__(32 * kTrainWarps) k_mlp_grad(const float* __re
                                                               const uint32_t* __restrict__ rows,
                                                               const float* __restrict__ labels, uint64_t n,
                                                               float inv_batch, float* __restrict__ grad,
-                                                              float* __restrict__ loss_sum, int given_dz) {
+                                                              float* __restrict__ loss_sum,
+                                                              const float* __restrict__ z,
+                                                              const VarianceSums* __restrict__ V, float eps) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainShared& S = *reinterpret_cast<TrainShared*>(smem_raw);
   load_mlp_shared(S.net, params);
@@ -1251,15 +1259,19 @@ __global__ void __launch_bounds__(32 * kTrainWarps) k_mlp_grad(const float* __re
     // binary cross-entropy when y is 0 or 1); dloss/dz = -y (1 - g) or g
     const float ya = va ? labels[ia] : 0.f, yb = vb ? labels[ib] : 0.f;
     auto dloss = [](float z, float y) { return y > 0.f ? -y * (1.f - sigmoidf_(z)) : sigmoidf_(z); };
-    // given_dz: the labels are dloss/dz already (the variance objective)
-    const float dza = va ? (given_dz ? ya : dloss(T.z3g, ya) * inv_batch) : 0.f;
-    const float dzb = vb ? (given_dz ? yb : dloss(T.z3g8, yb) * inv_batch) : 0.f;
+    // the variance objective: dL/dz from the batch's means and the rows' logits
+    auto variance_dz = [&](float zi, float x) {
+      const float gi = sigmoidf_(zi), h = eps + gi;
+      return gi * (1.f - gi) * (V->B - V->A * (x / h) * (x / h)) * inv_batch;
+    };
+    const float dza = va ? (V ? variance_dz(z[ia], ya) : dloss(T.z3g, ya) * inv_batch) : 0.f;
+    const float dzb = vb ? (V ? variance_dz(z[ib], yb) : dloss(T.z3g8, yb) * inv_batch) : 0.f;
     if (q == 0) {
       S.dz3[ra] = dza;
       S.dz3[rb] = dzb;
       auto softplus = [](float x) { return fmaxf(x, 0.f) + log1pf(expf(-fabsf(x))); };
       auto loss = [&](float z, float y) { return y > 0.f ? y * softplus(-z) : softplus(z); };
-      if (!given_dz) loss_acc += (va ? loss(T.z3g, ya) : 0.f) + (vb ? loss(T.z3g8, yb) : 0.f);
+      if (!V) loss_acc += (va ? loss(T.z3g, ya) : 0.f) + (vb ? loss(T.z3g8, yb) : 0.f);
     }
     // inputs and activations of the rows (bf16 values held as FP32), and
     // dz2 = dz3 W3 [z2 > 0]
@@ -1371,7 +1383,7 @@ __global__ void __launch_bounds__(32 * kTrainWarps) k_mlp_grad(const float* __re
   for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
   if (lane == 0) S.loss[warp] = loss_acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && !V) {
     float t = 0.f;
     for (int w = 0; w < kTrainWarps; w++) t += S.loss[w];
     atomicAdd(loss_sum, t);
@@ -1616,34 +1628,50 @@ tc_status launch_mlp_forward(const tc_mlp* M, const uint16_t* feat, const uint32
   return TC_OK;
 }
 
-// grad (device, kNParams) += gradient of the mean closure loss over rows;
-// *loss_sum (device) += summed per-row loss.  given_dz: labels hold dloss/dz3
-// per row and no loss is summed.
-tc_status launch_mlp_grad(const tc_mlp* M, const uint16_t* feat, const uint32_t* rows, const float* labels,
-                          uint64_t n, float* grad, float* loss_sum, cudaStream_t st, bool given_dz) {
-  if (!n) return TC_OK;
+// Blocks of the gradient launch: one 64-row tile each while they fit the GPU
+// at once (two per SM), then several tiles a block: each block ends with one
+// global atomic per parameter, which bound the launch of a block per tile
+// (100,003 rows: 58 us, and 74 us with up to eight blocks per SM).
+static tc_status launch_grad(const tc_mlp* M, const uint16_t* feat, const uint32_t* rows, const float* labels,
+                             uint64_t n, float* grad, float* loss_sum, const float* z, const VarianceSums* V, float eps,
+                             cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
     TC_CUDA(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainShared)));
     attr = true;
   }
-  k_mlp_grad<<<grid_cap(n, kTrainRows * TC_TRAIN_TILES), 32 * kTrainWarps, sizeof(TrainShared), st>>>(
-      M->params, reinterpret_cast<const __nv_bfloat16*>(feat), rows, labels, n, 1.0f / (float)n, grad, loss_sum,
-      given_dz ? 1 : 0);
+  static_assert(2 * (sizeof(TrainShared) + 1024) <= 227 * 1024, "two gradient blocks per SM");
+  const uint64_t tiles = (n + kTrainRows - 1) / kTrainRows, fit = (uint64_t)num_sms() * 2;
+  k_mlp_grad<<<(unsigned)(tiles < fit ? tiles : fit), 32 * kTrainWarps, sizeof(TrainShared), st>>>(
+      M->params, reinterpret_cast<const __nv_bfloat16*>(feat), rows, labels, n, 1.0f / (float)n, grad, loss_sum, z, V,
+      eps);
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());
   return TC_OK;
 }
 
-tc_status launch_variance_grad(const tc_mlp* M, const uint16_t* feat, const uint32_t* rows, const float* X,
-                               uint64_t n, float eps, float* grad, float* loss, float* z, float* dz,
-                               float* loss_scratch, cudaStream_t st) {
+// grad (device, kNParams) += gradient of the mean closure loss over rows;
+// *loss_sum (device) += summed per-row loss.
+tc_status launch_mlp_grad(const tc_mlp* M, const uint16_t* feat, const uint32_t* rows, const float* labels,
+                          uint64_t n, float* grad, float* loss_sum, cudaStream_t st) {
   if (!n) return TC_OK;
+  return launch_grad(M, feat, rows, labels, n, grad, loss_sum, nullptr, nullptr, 0.f, st);
+}
+
+size_t variance_scratch_bytes(uint64_t n) { return 256 + sizeof(float) * (n ? n : 1); }
+
+tc_status launch_variance_grad(const tc_mlp* M, const uint16_t* feat, const uint32_t* rows, const float* X,
+                               uint64_t n, float eps, float* grad, float* loss, void* scratch, cudaStream_t st) {
+  if (!n) return TC_OK;
+  static_assert(sizeof(VarianceSums) <= 256, "the logits follow");
+  VarianceSums* V = (VarianceSums*)scratch;
+  float* z = (float*)((char*)scratch + 256);
+  TC_CUDA(cudaMemsetAsync(V, 0, sizeof(*V), st));
   TC_TRY(launch_mlp_forward(M, feat, rows, n, z, st));
-  k_variance_dz<<<1, 1024, 0, st>>>(z, X, n, eps, dz, loss);
+  k_variance_sums<<<(unsigned)((n + kVarRows - 1) / kVarRows), kVarThreads, 0, st>>>(z, X, n, eps, V, loss);
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());
-  return launch_mlp_grad(M, feat, rows, dz, n, grad, loss_scratch, st, true);
+  return launch_grad(M, feat, rows, X, n, grad, loss, z, V, eps, st);
 }
 
 tc_status mlp_adam(tc_mlp* M, float lr, cudaStream_t st) {
