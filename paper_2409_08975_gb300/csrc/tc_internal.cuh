@@ -165,16 +165,14 @@ struct tc_graph {
   // independent of delta and of the motif: positions in the concatenated
   // lists where u's in-list and v's out-list reach time t (the first entry
   // with time >= t), and e's own position in v's in-list.
-  uint32_t* x_in;    // first position p in u's in-list with in_e[p].t >= t
-  uint32_t* x_out;   // first position p in v's out-list with out_e[p].t >= t
-  uint32_t* out2in;  // canonical position -> in-list position (inverse of in_eid)
-  // Range words of the anchors (tc::range_word): how far the anchor lies
-  // from the start and the end of its list, so that a window search needs
-  // no load of the list's offsets unless it runs beyond 65,534 entries.
-  uint32_t* r_in;    // x_in[e] in u's in-list
-  uint32_t* r_out;   // x_out[e] in v's out-list
-  uint32_t* r_o2i;   // out2in[e] in v's in-list
-  uint32_t* r_self;  // e itself in u's out-list
+  // Each carries its range word (tc::range_word), how far the anchor lies
+  // from the start and the end of its list, so that a window search needs no
+  // load of the list's offsets unless it runs beyond 65,534 entries: {anchor,
+  // range word} pairs, one 8-byte load.
+  uint2* x_in;       // first position p in u's in-list with in_e[p].t >= t
+  uint2* x_out;      // first position p in v's out-list with out_e[p].t >= t
+  uint2* out2in;     // canonical position -> in-list position (inverse of in_eid), in v's in-list
+  uint32_t* r_self;  // range word of e itself in u's out-list
 };
 
 namespace tc {

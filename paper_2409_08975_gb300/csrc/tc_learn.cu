@@ -130,7 +130,8 @@ constexpr uint32_t kFeatLut = 1024;
 struct FeatureArgs {
   const OutEdge* out_e;
   const uint32_t *out_off, *in_off, *out_t32, *in_t32, *pair_t32;
-  const uint32_t *x_in, *x_out, *out2in, *r_in, *r_out, *r_o2i, *r_self;
+  const uint2 *x_in, *x_out, *out2in;  // {anchor, range word}
+  const uint32_t* r_self;
   const PairSlot* table;
   uint32_t mask;
   int shift;
@@ -181,9 +182,9 @@ __global__ void __launch_bounds__(kFeatThreads) k_features32(const __grid_consta
     row[0] = log_count(w.y);
     row[1] = log_count(w.w);
     row[2] = __float2bfloat16_rn(log1pf((float)((uint64_t)w.y * (uint64_t)w.w)));
-    // entries of the list around anchor a (range word rw) with time in
-    // [lo, hi], and the list's length
-    auto degree = [&](const uint32_t* off, const uint32_t* t32, int32_t x, uint32_t a, uint32_t rw, uint32_t* total) {
+    // entries of the list around an anchor with time in [lo, hi], and the list's length
+    auto degree = [&](const uint32_t* off, const uint32_t* t32, int32_t x, uint2 anchor, uint32_t* total) {
+      const uint32_t a = anchor.x, rw = anchor.y;
       uint32_t s = a - (rw >> 16), f = a + (rw & 0xFFFFu);
       if ((rw >> 16) == kRangeCap) s = __ldg(off + x);
       if ((rw & 0xFFFFu) == kRangeCap) f = __ldg(off + x + 1);
@@ -192,10 +193,10 @@ __global__ void __launch_bounds__(kFeatThreads) k_features32(const __grid_consta
       return gallop<true, uint32_t>(s, f, a, hi, tt) - gallop<false, uint32_t>(s, f, a, lo, tt);
     };
     uint32_t in_u, out_u, in_v, out_v;
-    row[3] = log_count(degree(A.in_off, A.in_t32, e.x, __ldg(A.x_in + i), __ldg(A.r_in + i), &in_u));
-    row[4] = log_count(degree(A.out_off, A.out_t32, e.x, (uint32_t)i, __ldg(A.r_self + i), &out_u));
-    row[5] = log_count(degree(A.in_off, A.in_t32, e.y, __ldg(A.out2in + i), __ldg(A.r_o2i + i), &in_v));
-    row[6] = log_count(degree(A.out_off, A.out_t32, e.y, __ldg(A.x_out + i), __ldg(A.r_out + i), &out_v));
+    row[3] = log_count(degree(A.in_off, A.in_t32, e.x, __ldg(A.x_in + i), &in_u));
+    row[4] = log_count(degree(A.out_off, A.out_t32, e.x, make_uint2((uint32_t)i, __ldg(A.r_self + i)), &out_u));
+    row[5] = log_count(degree(A.in_off, A.in_t32, e.y, __ldg(A.out2in + i), &in_v));
+    row[6] = log_count(degree(A.out_off, A.out_t32, e.y, __ldg(A.x_out + i), &out_v));
     auto sigma = [&](uint32_t x, uint32_t y) -> uint32_t {
       uint32_t h = pair_slot(x, y, A.shift);
       for (uint64_t probe = 0; probe <= A.mask; probe++) {
@@ -1507,9 +1508,6 @@ tc_status launch_features(const tc_graph* g, const EdgeWin* win, int64_t delta, 
     A.x_in = g->x_in;
     A.x_out = g->x_out;
     A.out2in = g->out2in;
-    A.r_in = g->r_in;
-    A.r_out = g->r_out;
-    A.r_o2i = g->r_o2i;
     A.r_self = g->r_self;
     A.table = g->pair_hash;
     A.mask = g->hash_mask;

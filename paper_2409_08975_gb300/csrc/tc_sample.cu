@@ -78,12 +78,10 @@ struct WeightsArgs {
   const uint32_t* in_off;
   const uint32_t* out_t32;
   const uint32_t* in_t32;
-  const uint32_t* x_in;
-  const uint32_t* x_out;
-  const uint32_t* out2in;
-  const uint32_t* r_in;    // range words of x_in, x_out, out2in and of the edge in u's out-list
-  const uint32_t* r_out;
-  const uint32_t* r_o2i;
+  const uint2* x_in;  // anchors and their range words
+  const uint2* x_out;
+  const uint2* out2in;
+  // range word of the edge in u's out-list
   const uint32_t* r_self;
   int64_t tmin;
   uint64_t m;
@@ -129,10 +127,10 @@ __global__ void __launch_bounds__(kWThreads, TC_WEIGHTS_MIN_BLOCKS) k_weights(co
     // anchors: u's in-list (x_in) or the edge itself in u's out-list; the
     // edge itself in v's in-list (out2in) or v's out-list (x_out)
     if (A.alpha1 != 0)
-      side_window<Compact>(A, A.alpha1, A.beta1, e.src, A.alpha1 < 0 ? __ldg(A.x_in + i) : (uint32_t)i, e.t, &lo1,
+      side_window<Compact>(A, A.alpha1, A.beta1, e.src, A.alpha1 < 0 ? __ldg(&A.x_in[i].x) : (uint32_t)i, e.t, &lo1,
                            &hi1);
     if (A.alpha3 != 0)
-      side_window<Compact>(A, A.alpha3, A.beta3, e.dst, A.alpha3 < 0 ? __ldg(A.out2in + i) : __ldg(A.x_out + i), e.t,
+      side_window<Compact>(A, A.alpha3, A.beta3, e.dst, A.alpha3 < 0 ? __ldg(&A.out2in[i].x) : __ldg(&A.x_out[i].x), e.t,
                            &lo3, &hi3);
     EdgeWin r;
     r.lo1 = lo1;
@@ -173,8 +171,8 @@ __global__ void __launch_bounds__(kWThreads, TC_WEIGHTS_MIN_BLOCKS) k_weights(co
 // The vertex x (the edge's source, or its destination when dst_side) is
 // read from the edge record only then.
 __device__ __forceinline__ void side_window_rw(const WeightsArgs& A, int alpha, int beta, uint64_t i, bool dst_side,
-                                               uint32_t a, uint32_t rw, bool exact, int64_t t, uint32_t* lo,
-                                               uint32_t* hi) {
+                                               uint2 anchor, bool exact, int64_t t, uint32_t* lo, uint32_t* hi) {
+  const uint32_t a = anchor.x, rw = anchor.y;
   const uint32_t* off = alpha < 0 ? A.in_off : A.out_off;
   uint32_t s = a - (rw >> 16), f = a + (rw & 0xFFFFu);
   if ((rw >> 16) == kRangeCap || (rw & 0xFFFFu) == kRangeCap) {
@@ -218,13 +216,13 @@ __global__ void __launch_bounds__(kWThreads, TC_WEIGHTS_MIN_BLOCKS)
     // anchors: u's in-list (x_in, exact) or the edge itself in u's out-list;
     // the edge itself in v's in-list (out2in) or v's out-list (x_out, exact)
     if (A.alpha1 < 0)
-      side_window_rw(A, -1, A.beta1, i, false, __ldg(A.x_in + i), __ldg(A.r_in + i), true, t, &lo1, &hi1);
+      side_window_rw(A, -1, A.beta1, i, false, __ldg(A.x_in + i), true, t, &lo1, &hi1);
     else if (A.alpha1 > 0)
-      side_window_rw(A, 1, A.beta1, i, false, (uint32_t)i, __ldg(A.r_self + i), false, t, &lo1, &hi1);
+      side_window_rw(A, 1, A.beta1, i, false, make_uint2((uint32_t)i, __ldg(A.r_self + i)), false, t, &lo1, &hi1);
     if (A.alpha3 < 0)
-      side_window_rw(A, -1, A.beta3, i, true, __ldg(A.out2in + i), __ldg(A.r_o2i + i), false, t, &lo3, &hi3);
+      side_window_rw(A, -1, A.beta3, i, true, __ldg(A.out2in + i), false, t, &lo3, &hi3);
     else if (A.alpha3 > 0)
-      side_window_rw(A, 1, A.beta3, i, true, __ldg(A.x_out + i), __ldg(A.r_out + i), true, t, &lo3, &hi3);
+      side_window_rw(A, 1, A.beta3, i, true, __ldg(A.x_out + i), true, t, &lo3, &hi3);
     __stcs(reinterpret_cast<uint4*>(A.win + i), make_uint4(lo1, hi1 - lo1, lo3, hi3 - lo3));
     const unsigned long long wv = (unsigned long long)(hi1 - lo1) * (unsigned long long)(hi3 - lo3);
     __stcs(reinterpret_cast<unsigned long long*>(A.w + i), wv);
@@ -286,9 +284,6 @@ tc_status launch_weights_scan(const tc_graph* g, const Plan& plan, int64_t delta
   A.x_in = g->x_in;
   A.x_out = g->x_out;
   A.out2in = g->out2in;
-  A.r_in = g->r_in;
-  A.r_out = g->r_out;
-  A.r_o2i = g->r_o2i;
   A.r_self = g->r_self;
   A.tmin = g->tmin;
   A.m = m;

@@ -157,3 +157,20 @@ def test_features_of_32_and_64_bit_times_are_the_same(tc, name, m, delta):
         assert w.W > 0 or delta == 0
         rows.append(tc.tc_edge_features(g, tc.make_motif(CHORD, window=1), delta * scale, w).view(torch.int16))
     assert torch.equal(rows[0], rows[1])
+
+
+@pytest.mark.parametrize("n,m,span", [(1, 1, 1), (2, 2, 1), (3, 4095, 5), (3, 4096, 1), (70_000, 4097, 1 << 20),
+                                      (300, 40_961, (1 << 32) - 1), (5000, 9000, 1 << 32), (1 << 22, 50_000, 1 << 31)])
+def test_lists_of_both_time_widths(tc, n, m, span):
+    # record sorts (spans below 2^32) and pair sorts at tile edges, with one
+    # vertex, one time, ties, and up to three digit passes, against the oracle
+    import torch
+    import oracle
+    from test_gpu_parity import _check_csr
+    rng = np.random.default_rng(m)
+    s, d = rng.integers(0, n, m).astype(np.int32), rng.integers(0, n, m).astype(np.int32)
+    t = rng.integers(0, span, m).astype(np.int64) - 7
+    t[0], t[-1] = -7, span - 7  # the whole span, negative times included
+    dev = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=dt)  # noqa: E731
+    g = tc.tc_build_temporal_csr(n, dev(s, torch.int32), dev(d, torch.int32), dev(t, torch.int64))
+    _check_csr(tc, g, oracle.build_csr(n, s, d, t))
