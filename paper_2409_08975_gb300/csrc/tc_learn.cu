@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -118,7 +119,8 @@ __global__ void __launch_bounds__(256) k_features(const OutEdge* __restrict__ ou
 // four degree windows are galloping searches from the window anchors, whose
 // range words also tell the total degrees, where k_features bisects the whole
 // lists on their 16-byte records.  A block lists the edges with w > 0 of its
-// tile of kFeatTile (fewer than half) and runs full warps of those, and takes
+// tile (kFeatTile edges, fewer on small graphs so that every SM gets some) and
+// runs full warps of those, fewer than half of all, and takes
 // log1p of a count below kFeatLut from a table that it fills with the same
 // function.  Bound by the latency of the searches and the two random hash
 // probes per edge (ncu: long-scoreboard stalls 21 of 30 cycles, DRAM 38%): 20M
@@ -138,6 +140,7 @@ struct FeatureArgs {
   const EdgeWin* win;
   uint64_t m;
   int64_t tmin, delta;
+  uint32_t tile;  // a multiple of kFeatThreads, at most kFeatTile
   __nv_bfloat16* feat;
 };
 
@@ -148,10 +151,10 @@ __global__ void __launch_bounds__(kFeatThreads) k_features32(const __grid_consta
   for (uint32_t c = threadIdx.x; c < kFeatLut; c += kFeatThreads) lut[c] = __float2bfloat16_rn(log1pf((float)c));
   if (threadIdx.x == 0) nlive = 0;
   __syncthreads();
-  const uint64_t base = (uint64_t)blockIdx.x * kFeatTile;
+  const uint64_t base = (uint64_t)blockIdx.x * A.tile;
   const int lane = threadIdx.x & 31;
 #pragma unroll 1
-  for (uint32_t r = threadIdx.x; r < kFeatTile; r += kFeatThreads) {  // whole warps: kFeatTile is a multiple
+  for (uint32_t r = threadIdx.x; r < A.tile; r += kFeatThreads) {  // whole warps
     bool is = false;
     if (base + r < A.m) {
       const uint4 w = __ldg(reinterpret_cast<const uint4*>(A.win + base + r));
@@ -1517,7 +1520,8 @@ tc_status launch_features(const tc_graph* g, const EdgeWin* win, int64_t delta, 
     A.tmin = g->tmin;
     A.delta = delta;
     A.feat = reinterpret_cast<__nv_bfloat16*>(feat);
-    k_features32<<<(unsigned)((m + kFeatTile - 1) / kFeatTile), kFeatThreads, 0, st>>>(A);
+    A.tile = (uint32_t)std::min<uint64_t>(kFeatTile, (m / ((uint64_t)num_sms() * 8) / kFeatThreads + 1) * kFeatThreads);
+    k_features32<<<(unsigned)((m + A.tile - 1) / A.tile), kFeatThreads, 0, st>>>(A);
     TC_LAUNCHED(1);
     TC_CUDA(cudaGetLastError());
     return TC_OK;

@@ -802,7 +802,8 @@ __device__ __forceinline__ void block_commit(SampleSums* G, uint64_t W, uint64_t
 // CheckMotif over all paths is the exact count C, the sum of squares gives
 // the exact variance of one sample.
 //
-// A warp takes runs of kPathRun consecutive paths, lane l every 32nd of them
+// A warp takes runs of consecutive paths (4096, fewer where W would leave warps
+// without one: 20,000 edges, 276 us in runs of 4096), lane l every 32nd of them
 // from l on: the middle edge and its windows, and the end edge e1, are loaded
 // when a lane crosses into the next one (an edge has thousands of paths where
 // an exact count takes long), and the pair (p1, p3) is stepped on, so that a
@@ -811,10 +812,10 @@ __device__ __forceinline__ void block_commit(SampleSums* G, uint64_t W, uint64_t
 // graph: 26.2 ms (41.2 ms with a CDF search, a 64-bit division and both end
 // loads per path; 28.5 ms without pair_window's look at the list's ends).
 // Four blocks of 256 (64 registers): with five 29.9 ms, with six 33.9 ms.
-constexpr uint64_t kPathRun = 4096;
+constexpr uint64_t kPathRun = 4096;  // a multiple of 32
 template <bool Compact>
 __global__ void __launch_bounds__(256, 4) k_path_sum(const __grid_constant__ SamplerArgs A,
-                                                    const __grid_constant__ Plan P) {
+                                                    const __grid_constant__ Plan P, uint64_t length) {
   typedef SampleTime<Compact> Tm;
   const IndexHeader* H = A.hdr;
   const uint64_t W = H->W;
@@ -835,8 +836,8 @@ __global__ void __launch_bounds__(256, 4) k_path_sum(const __grid_constant__ Sam
   const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   uint64_t hits = 0, checked = 0;  // a thread may take more than 2^32 paths
-  for (uint64_t run = warp * kPathRun; run < W; run += warps * kPathRun) {
-    const uint64_t end = W - run < kPathRun ? W : run + kPathRun;
+  for (uint64_t run = warp * length; run < W; run += warps * length) {
+    const uint64_t end = W - run < length ? W : run + length;
     uint64_t stop = 0;  // end of the paths of the current middle edge
     uint32_t lo1 = 0, lo3 = 0, d3 = 1, i1 = 0, i3 = 0;
     int32_t u = 0, v = 0, up = 0, vp = 0;
@@ -1666,7 +1667,8 @@ tc_status launch_path_sum(const tc_graph* g, const Plan& plan, int64_t delta, co
   uint64_t blocks = (uint64_t)num_sms() * (bps > 0 ? bps : 1);
   const uint64_t need = (W + 255) / 256;
   if (need < blocks) blocks = need ? need : 1;
-  kernel<<<(unsigned)blocks, 256, 0, st>>>(A, plan);
+  const uint64_t share = W / (blocks * (256 / 32)) & ~31ull;  // paths per warp
+  kernel<<<(unsigned)blocks, 256, 0, st>>>(A, plan, std::max<uint64_t>(32, std::min(share, kPathRun)));
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());
   return TC_OK;
