@@ -272,7 +272,7 @@ tc_status create(const tc_query* hq, int64_t nq, const tc_batch_options* opts, c
       max_m = std::max<uint64_t>(max_m, (uint64_t)S.g->m);
     }
     Q.slot = it->second;
-    const uint64_t chunk = Q.q.k >= kBatchOrderedMinSamples ? kChunkSamples : Q.q.k;
+    const uint64_t chunk = Q.q.k >= kBatchOrderedMinSamples ? kSmallChunkSamples : Q.q.k;
     for (uint64_t base = 0; base < Q.q.k; base += chunk) {
       Record R{(int)i, base, std::min<uint64_t>(Q.q.k - base, chunk), nullptr};
       if (Q.q.k >= kBatchOrderedMinSamples) {

@@ -1018,12 +1018,14 @@ __device__ __forceinline__ void sample_one(const SamplerArgs& A, const Plan& P, 
 // overflow word is set and the sampler takes the chunk in id order instead:
 // the sums are integers and do not depend on the order.
 //
-// Measured for 1e9 samples of the 300M-edge graph (chunks of 2^28): order
-// passes 7.3 ms (4.1 + 3.2) and sampler 29.5 ms, where two counting passes
-// over 16-bit keys with their histograms and scans took 12.4 ms and the
-// sampler on that order 52.6 ms.  A sampler on the order by 20, 24 or 32 bits
-// of the draw, otherwise unchanged, took 43.5, 38.7 and 39.0 ms: beyond 24
-// bits (the bucket and its bins here) nothing more is gained.
+// Measured for 1e9 samples of the 300M-edge graph: order passes 7.3 ms (4.1 +
+// 3.2) and sampler 24.3 ms, where two counting passes over 16-bit keys with
+// their histograms and scans took 12.4 ms and the sampler on that order 52.6
+// ms.  A sampler on the order by 20, 24 or 32 bits of the draw, otherwise
+// unchanged, took 43.5, 38.7 and 39.0 ms: beyond 24 bits (the bucket and its
+// bins here) nothing more is gained.  Chunks are as large as memory allows (up
+// to 2^30): each chunk reads the graph once from DRAM, and in chunks of 2^28
+// the sampler took 28.9 ms.
 constexpr int kOrderThreads = 512;
 constexpr int kOrderItems = 16;
 constexpr int kOrderTile = kOrderThreads * kOrderItems;  // 8192
@@ -1614,16 +1616,23 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
     timer.stop();
     return s;
   }
-  // samples in chunks, each with an order of its own
-  const uint64_t chunk = k < kChunkSamples ? k : kChunkSamples;
+  // samples in chunks, each with an order of its own (about 11 bytes a sample;
+  // smaller chunks when the memory for a large one is not there)
   const uint32_t wave = (uint32_t)max_blocks;
-  const size_t sbytes = order_scratch_bytes(chunk, wave);
+  uint64_t chunk = std::min(k, kChunkSamples);
+  size_t scratch = 0;
   char* buf = nullptr;
-  // the last chunk is smaller than the others, but its order may hold more rounding
-  const uint64_t tail = k % chunk;
-  const size_t obytes = std::max(order_bytes(chunk, wave), tail ? order_bytes(tail, wave) : (size_t)0);
-  const size_t scratch = std::max(sbytes, tail ? order_scratch_bytes(tail, wave) : (size_t)0);
-  TC_CUDA(pool_malloc(&buf, scratch + obytes, st));
+  for (;;) {
+    // the last chunk is smaller than the others, but its order may hold more rounding
+    const uint64_t tail = k % chunk;
+    scratch = std::max(order_scratch_bytes(chunk, wave), tail ? order_scratch_bytes(tail, wave) : (size_t)0);
+    const size_t obytes = std::max(order_bytes(chunk, wave), tail ? order_bytes(tail, wave) : (size_t)0);
+    const cudaError_t e = pool_malloc(&buf, scratch + obytes, st);
+    if (e == cudaSuccess) break;
+    if (e != cudaErrorMemoryAllocation || chunk <= kSmallChunkSamples) return cuda_status(e, "pool_malloc(order)");
+    cudaGetLastError();
+    chunk = std::max(chunk / 2, kSmallChunkSamples);
+  }
   void* order = buf + scratch;
   tc_status s = TC_OK;
   for (uint64_t base = 0; base < k && s == TC_OK; base += chunk) {

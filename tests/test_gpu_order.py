@@ -174,3 +174,18 @@ def test_lists_of_both_time_widths(tc, n, m, span):
     dev = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=dt)  # noqa: E731
     g = tc.tc_build_temporal_csr(n, dev(s, torch.int32), dev(d, torch.int32), dev(t, torch.int64))
     _check_csr(tc, g, oracle.build_csr(n, s, d, t))
+
+
+def test_chunks_of_2_30_samples(tc):
+    # one call over a chunk bound against its parts, which are ordered apart
+    g = graph(tc, "bursty")
+    mot = tc.make_motif(C4)
+    w = tc.tc_path_weights(g, mot, 3600)
+    parts = [1 << 29, 1 << 29, 600_077]
+    whole = tc.tc_sample_estimate(g, mot, 3600, w, sum(parts), 5, 9)
+    total = dict(sum_x=0, sum_x2=0, hits=0, checked=0)
+    for i, k in enumerate(parts):
+        e = tc.tc_sample_estimate(g, mot, 3600, w, k, 5, 9 + sum(parts[:i]))
+        for key in total:
+            total[key] += e[key]
+    assert {key: whole[key] for key in total} == total
