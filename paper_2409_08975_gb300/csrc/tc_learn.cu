@@ -816,17 +816,24 @@ __device__ __forceinline__ void tc05_fence_before() { asm volatile("tcgen05.fenc
 __device__ __forceinline__ void tc05_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// 16 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
+// Starts the load of 16 consecutive FP32 columns of this thread's TMEM lane;
+// the values are there after tmem_wait.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+}
+// Waits for this thread's TMEM loads; the registers pass through a second,
+// empty statement, so that no use (or copy) of them moves before the wait.
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int j = 0; j < 16; j++) v[j] = __uint_as_float(r[j]);
+  asm volatile(""
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
 }
 
 struct alignas(1024) UmmaShared {
@@ -843,19 +850,18 @@ struct alignas(1024) UmmaShared {
   uint32_t err;
   unsigned long long red[4];
   uint32_t wcnt[4];                          // rows with w > 0 in each warp's quarter of the tile
-  unsigned long long pre[16 * kUmmaM + 1];   // the tile's prefix entries (proposal)
   uint16_t live[16 * kUmmaM];                // the tile's rows with w > 0, in order (proposal)
 };
-// At least 30 KB of shared memory per block, so that at most seven blocks
-// share an SM (8 x 31 KB exceeds the SM's 228 KB): their TMEM (kTmemCols
-// each) then always fits the 512 columns of an SM and no allocation waits.
+// At least 32 KB of shared memory per block, so that at most six blocks share
+// an SM (7 x 33 KB exceeds the SM's 228 KB): their TMEM (kTmemCols each) then
+// always fits the 512 columns of an SM and no allocation waits.
 constexpr size_t kUmmaSmemBytes =
-    sizeof(UmmaShared) + 1024 > 30 * 1024 ? sizeof(UmmaShared) + 1024 : 30 * 1024;
-static_assert(7 * kTmemCols <= 512, "TMEM of the blocks one SM can hold");
-static_assert(kUmmaSmemBytes * 4 <= 227 * 1024, "four blocks per SM");
+    sizeof(UmmaShared) + 1024 > 32 * 1024 ? sizeof(UmmaShared) + 1024 : 32 * 1024;
+static_assert(6 * kTmemCols <= 512, "TMEM of the blocks one SM can hold");
+static_assert((kUmmaSmemBytes + 1024) * 6 <= 228 * 1024, "six blocks per SM");
 constexpr int kUmmaSubTiles = 16;                         // 128-row sub-tiles per tile
 constexpr uint64_t kUmmaTile = kUmmaSubTiles * kUmmaM;     // 2048 rows: the scan's tile
-constexpr int kUmmaBlocksPerSm = 4;                        // resident blocks (launch bounds, shared memory)
+constexpr int umma_blocks_per_sm(bool proposal) { return proposal ? 6 : 4; }  // resident blocks (see k_mlp_umma)
 constexpr uint64_t kUmmaWaitNs = 1000000000ull;            // bound of each completion wait: 1 s
 
 __device__ __forceinline__ uint64_t global_ns() {
@@ -878,11 +884,16 @@ __device__ __forceinline__ bool umma_wait(uint64_t* mbar, uint32_t parity) {
 // For the rows of the tiles this block takes (rows[i] or i index the
 // feature rows), the logits (Proposal = false: into logits), or (Proposal =
 // true) h, q = w h and each 2048-row tile's sum of q as k_proposal computes
-// them: the tile's prefix entries are staged in shared memory, the rows with
-// w > 0 listed in order, and only those go through the network, 128 to a
-// sub-tile (rows with w = 0 get h = 1, q = 0).
+// them: the rows with w > 0 of a tile are listed in order, and only those go
+// through the network, 128 to a sub-tile (rows with w = 0 get h = 1, q = 0).
+//
+// Bound by the latency of a sub-tile's chain (stage, MMA, epilogue, MMA,
+// epilogue) and by shared memory (half of its bandwidth), so by blocks per SM:
+// 1e8 edges take 2.30 ms with six blocks, 2.52 with five; with the tile's
+// prefix entries staged in shared memory, which left room for four, 2.52 ms.
+// The logits of whole row sets do not gain from more than four (1e6 rows 40 us).
 template <bool Proposal>
-__global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const float* __restrict__ params,
+__global__ void __launch_bounds__(kUmmaM, umma_blocks_per_sm(Proposal)) k_mlp_umma(const float* __restrict__ params,
                                                       const __nv_bfloat16* __restrict__ feat,
                                                       const uint32_t* __restrict__ rows, uint64_t n,
                                                       float* __restrict__ logits, const uint64_t* __restrict__ prefix,
@@ -935,26 +946,33 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
     // or the rows with w > 0, listed in order (proposal)
     uint32_t nrun = trows;
     if (Proposal) {
-      __syncthreads();  // the previous tile's lists are consumed
-      for (uint32_t i = tid; i <= trows; i += kUmmaM) S.pre[i] = __ldg(prefix + base + i);
-      __syncthreads();
-      const uint32_t q0 = (uint32_t)warp * (kUmmaTile / 4);  // this warp's quarter of the tile
-      uint32_t cnt = 0;
-      for (uint32_t r = 0; r < kUmmaTile / 4; r += 32) {
-        const uint32_t row = q0 + r + lane;
-        const bool live = row < trows && S.pre[row + 1] != S.pre[row];
-        cnt += __popc(__ballot_sync(0xffffffffu, live));
+      // this warp's quarter of the tile: which rows are live (kept as one
+      // ballot per 32 rows), the others' h = 1 and q = 0 (as k_proposal)
+      constexpr int kRounds = kUmmaTile / 4 / 32;
+      const uint32_t q0 = (uint32_t)warp * (kUmmaTile / 4) + lane;
+      uint32_t masks[kRounds], cnt = 0;
+#pragma unroll
+      for (int r = 0; r < kRounds; r++) {
+        const uint32_t row = q0 + 32 * r;
+        bool live = false;
+        if (row < trows) {
+          live = __ldg(prefix + base + row + 1) != __ldg(prefix + base + row);
+          if (!live) {
+            q[base + row] = 0;
+            h[base + row] = 1;
+          }
+        }
+        masks[r] = __ballot_sync(0xffffffffu, live);
+        cnt += __popc(masks[r]);
       }
       if (lane == 0) S.wcnt[warp] = cnt;
-      __syncthreads();
+      __syncthreads();  // (the previous tile's list is consumed: its last sub-tile ended in a barrier)
       uint32_t at = 0;
       for (int v = 0; v < warp; v++) at += S.wcnt[v];
-      for (uint32_t r = 0; r < kUmmaTile / 4; r += 32) {
-        const uint32_t row = q0 + r + lane;
-        const bool live = row < trows && S.pre[row + 1] != S.pre[row];
-        const uint32_t mask = __ballot_sync(0xffffffffu, live);
-        if (live) S.live[at + __popc(mask & ((1u << lane) - 1u))] = (uint16_t)row;
-        at += __popc(mask);
+#pragma unroll
+      for (int r = 0; r < kRounds; r++) {
+        if ((masks[r] >> lane) & 1u) S.live[at + __popc(masks[r] & ((1u << lane) - 1u))] = (uint16_t)(q0 + 32 * r);
+        at += __popc(masks[r]);
       }
       nrun = S.wcnt[0] + S.wcnt[1] + S.wcnt[2] + S.wcnt[3];
       __syncthreads();
@@ -962,24 +980,29 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
     unsigned long long tsum = 0;
     // this thread's feature row of a sub-tile (zero past the rows to run); the
     // next sub-tile's row is loaded while the current one is on the tensor cores
-    auto fetch = [&](uint32_t at, uint4& lo, uint4& hi) {
+    // (with it, for the proposal, its weight w)
+    auto fetch = [&](uint32_t at, uint4& lo, uint4& hi, unsigned long long& wgt) {
       lo = hi = make_uint4(0, 0, 0, 0);
+      wgt = 0;
       if (at < nrun) {
         const uint64_t r = base + (Proposal ? (uint32_t)S.live[at] : at);
         const uint4* src = reinterpret_cast<const uint4*>(feat + (uint64_t)(rows ? rows[r] : r) * kF);
         lo = __ldg(src);
         hi = __ldg(src + 1);
+        if (Proposal) wgt = __ldg(prefix + r + 1) - __ldg(prefix + r);
       }
     };
     uint4 nlo, nhi;
-    fetch(tid, nlo, nhi);
+    unsigned long long nw;
+    fetch(tid, nlo, nhi, nw);
     for (uint32_t r0 = 0; r0 < nrun && ok; r0 += kUmmaM) {  // 128-row sub-tiles
       const uint32_t idx = r0 + tid;
       const bool valid = idx < nrun;
       const uint32_t local = Proposal ? (valid ? (uint32_t)S.live[idx] : 0u) : idx;
       const uint64_t row = base + local;
       const uint4 xlo = nlo, xhi = nhi;
-      fetch(idx + kUmmaM, nlo, nhi);
+      const unsigned long long wv = nw;  // > 0 for a listed row
+      fetch(idx + kUmmaM, nlo, nhi, nw);
       *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.A1) + umma_offset(tid, 0, kF)) = xlo;
       *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.A1) + umma_offset(tid, 8, kF)) = xhi;
       fence_async_smem();
@@ -996,17 +1019,21 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
       if (!ok) break;  // parity stays that of the phase still pending
       parity ^= 1;
       tc05_fence_after();
+      // (the next 16 columns are on their way while these are used)
+      uint32_t acc[2][16];
+      tmem_ld16(tmem + lane_addr, acc[0]);
 #pragma unroll
       for (int c = 0; c < 4; c++) {  // bias, ReLU, bf16: the A operand of layer 2
-        float v[16];
-        tmem_ld16(tmem + lane_addr + (uint32_t)(c * 16), v);
+        tmem_wait(acc[c & 1]);
+        if (c < 3) tmem_ld16(tmem + lane_addr + (uint32_t)(c * 16 + 16), acc[(c + 1) & 1]);
+        auto v = [&](int j) { return __uint_as_float(acc[c & 1][j]); };
         float b[16];  // the bias as four 16-byte shared loads
 #pragma unroll
         for (int j = 0; j < 4; j++)
           *reinterpret_cast<float4*>(b + 4 * j) = reinterpret_cast<const float4*>(S.b1)[c * 4 + j];
         uint32_t pk[8];
 #pragma unroll
-        for (int j = 0; j < 8; j++) pk[j] = relu_bf16x2(v[2 * j] + b[2 * j], v[2 * j + 1] + b[2 * j + 1]);
+        for (int j = 0; j < 8; j++) pk[j] = relu_bf16x2(v(2 * j) + b[2 * j], v(2 * j + 1) + b[2 * j + 1]);
         char* dst = reinterpret_cast<char*>(S.A2);
         *reinterpret_cast<uint4*>(dst + umma_offset(tid, c * 16, kH)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(dst + umma_offset(tid, c * 16 + 8, kH)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
@@ -1029,10 +1056,13 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
       parity ^= 1;
       tc05_fence_after();
       float z = S.b3;  // layer 3 in FP32 on the bf16-rounded activations
+      tmem_ld16(tmem + lane_addr, acc[0]);
 #pragma unroll
       for (int c = 0; c < 4; c++) {
-        float v[16], b[16], w3[16];
-        tmem_ld16(tmem + lane_addr + (uint32_t)(c * 16), v);
+        tmem_wait(acc[c & 1]);
+        if (c < 3) tmem_ld16(tmem + lane_addr + (uint32_t)(c * 16 + 16), acc[(c + 1) & 1]);
+        auto v = [&](int j) { return __uint_as_float(acc[c & 1][j]); };
+        float b[16], w3[16];
 #pragma unroll
         for (int j = 0; j < 4; j++) {
           *reinterpret_cast<float4*>(b + 4 * j) = reinterpret_cast<const float4*>(S.b2)[c * 4 + j];
@@ -1040,7 +1070,7 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
         }
 #pragma unroll
         for (int j = 0; j < 8; j++) {  // ReLU and bf16 rounding of a pair in one instruction, then widened
-          const uint32_t pk = relu_bf16x2(v[2 * j] + b[2 * j], v[2 * j + 1] + b[2 * j + 1]);
+          const uint32_t pk = relu_bf16x2(v(2 * j) + b[2 * j], v(2 * j + 1) + b[2 * j + 1]);
           z = fmaf(__uint_as_float(pk << 16), w3[2 * j], z);
           z = fmaf(__uint_as_float(pk & 0xFFFF0000u), w3[2 * j + 1], z);
         }
@@ -1050,7 +1080,6 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
         if (!Proposal) {
           logits[row] = z;
         } else {
-          const unsigned long long wv = S.pre[local + 1] - S.pre[local];  // > 0: a listed row
           const float fv = floorf(scale * (eps + sigmoidf_(z)) + 0.5f);
           const uint32_t hv = fv < 1.f ? 1u : (uint32_t)fv;
           hlo = hv < hlo ? hv : hlo;
@@ -1065,12 +1094,6 @@ __global__ void __launch_bounds__(kUmmaM, kUmmaBlocksPerSm) k_mlp_umma(const flo
       }
     }
     if (Proposal && ok) {
-      // rows with w = 0 are never drawn: h = 1, q = 0 (as k_proposal)
-      for (uint32_t r = tid; r < trows; r += kUmmaM)
-        if (S.pre[r + 1] == S.pre[r]) {
-          q[base + r] = 0;
-          h[base + r] = 1;
-        }
       // the tile's sum of q
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -1604,10 +1627,10 @@ static tc_status launch_umma(const tc_mlp* M, const uint16_t* feat, const uint32
                                  (int)kUmmaSmemBytes));
     attr = true;
   }
-  // kUmmaBlocksPerSm blocks per SM: what the launch bounds' registers and the
+  // umma_blocks_per_sm blocks per SM: what the launch bounds' registers and the
   // shared memory allow (their TMEM, 64 columns each, fits an SM's 512)
   const uint64_t T = Proposal ? (n + kUmmaTile - 1) / kUmmaTile : (n + kUmmaM - 1) / kUmmaM;
-  uint64_t blocks = (uint64_t)num_sms() * kUmmaBlocksPerSm;
+  uint64_t blocks = (uint64_t)num_sms() * umma_blocks_per_sm(Proposal);
   if (blocks > T) blocks = T;
   k_mlp_umma<Proposal><<<(unsigned)blocks, kUmmaM, kUmmaSmemBytes, st>>>(
       M->params, reinterpret_cast<const __nv_bfloat16*>(feat), rows, n, logits, prefix, eps, scale, h, q, tile_sums,
