@@ -48,6 +48,39 @@ cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+namespace {
+constexpr size_t kPinnedBytes = 128 << 10;
+struct PinnedBuffer {
+  void* p = nullptr;
+  ~PinnedBuffer() {
+    if (p) cudaFreeHost(p);
+  }
+};
+thread_local PinnedBuffer t_pinned;
+}  // namespace
+
+cudaError_t read_back(void* host, const void* device, size_t bytes, cudaStream_t st) {
+  void* to = host;
+  if (bytes <= kPinnedBytes) {
+    if (t_pinned.p) {  // a device reset takes the buffer with it
+      cudaPointerAttributes a;
+      if (cudaPointerGetAttributes(&a, t_pinned.p) != cudaSuccess || a.type != cudaMemoryTypeHost) {
+        cudaGetLastError();
+        t_pinned.p = nullptr;
+      }
+    }
+    if (!t_pinned.p && cudaHostAlloc(&t_pinned.p, kPinnedBytes, cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      t_pinned.p = nullptr;
+    }
+    if (t_pinned.p) to = t_pinned.p;
+  }
+  cudaError_t e = cudaMemcpyAsync(to, device, bytes, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && to != host) std::memcpy(host, to, bytes);
+  return e;
+}
+
 tc_status set_error(tc_status st, const std::string& msg) {
   t_err = msg;
   return st;
@@ -437,10 +470,13 @@ tc_status tc_path_weights(const tc_graph* g, const tc_motif* motif, int64_t delt
   it.stop();
   uint32_t h_err = 0;
   if (s == TC_OK && h_W) {
-    e = cudaMemcpyAsync(h_W, d_prefix + m, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    IndexHeader h;  // written by the guide kernel: W = prefix[m] and the error bits so far
+    e = read_back(&h, d_index, sizeof(h), st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_path_weights");
+    if (s == TC_OK) {
+      *h_W = h.W;
+      h_err = h.status;
+    }
   }
   cudaFreeAsync(scratch, st);
   if (s == TC_OK && h_err) s = device_status(h_err, "tc_path_weights");
@@ -466,8 +502,7 @@ static tc_status sample_common(const tc_graph* g, const tc_motif* motif, int64_t
   SampleSums h;
   std::memset(&h, 0, sizeof(h));
   if (s == TC_OK) {
-    e = cudaMemcpyAsync(&h, sums, sizeof(h), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = read_back(&h, sums, sizeof(h), st);
     if (e != cudaSuccess) s = cuda_status(e, what);
   }
   cudaFreeAsync(sums, st);
@@ -555,8 +590,7 @@ tc_status tc_exact_count(const tc_graph* g, const tc_motif* motif, int64_t delta
   if (((uintptr_t)d_index & 255) != 0) return set_error(TC_ERR_INVALID_ARG, "index must be 256-byte aligned");
   cudaStream_t st = S(stream);
   uint64_t W = 0;
-  TC_CUDA(cudaMemcpyAsync(&W, d_prefix + g->m, sizeof(W), cudaMemcpyDeviceToHost, st));
-  TC_CUDA(cudaStreamSynchronize(st));
+  TC_CUDA(read_back(&W, d_prefix + g->m, sizeof(W), st));
   SampleSums* sums = nullptr;
   TC_CUDA(pool_malloc(&sums, sizeof(SampleSums), st));
   tc_status s = TC_OK;
@@ -566,8 +600,7 @@ tc_status tc_exact_count(const tc_graph* g, const tc_motif* motif, int64_t delta
   SampleSums h;
   std::memset(&h, 0, sizeof(h));
   if (s == TC_OK) {
-    e = cudaMemcpyAsync(&h, sums, sizeof(h), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = read_back(&h, sums, sizeof(h), st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_exact_count");
   }
   cudaFreeAsync(sums, st);
@@ -591,8 +624,7 @@ tc_status tc_exact_count(const tc_graph* g, const tc_motif* motif, int64_t delta
 static tc_status check_index_header(const tc_graph* g, const Plan& plan, int64_t delta, const void* d_index,
                                     cudaStream_t st) {
   IndexHeader h;
-  TC_CUDA(cudaMemcpyAsync(&h, d_index, sizeof(h), cudaMemcpyDeviceToHost, st));
-  TC_CUDA(cudaStreamSynchronize(st));
+  TC_CUDA(read_back(&h, d_index, sizeof(h), st));
   const bool ok = h.magic == kIndexMagic && h.graph_id == g->id && h.delta == delta && h.cls[0] == plan.alpha1 &&
                   h.cls[1] == plan.alpha3 && h.cls[2] == plan.beta1 && h.cls[3] == plan.beta3 &&
                   h.closed == plan.closed && h.anchor[0] == plan.e1 && h.anchor[1] == plan.mid &&
@@ -658,18 +690,18 @@ tc_status tc_sample_features(const tc_graph* g, const tc_motif* motif, int64_t d
   if (s == TC_OK && n_samples)
     s = launch_sampler(g, plan, delta, d_prefix, d_index, n_samples, seed, sample_offset, trace, sums, st);
   if (s == TC_OK) s = launch_sample_features(g, d_prefix, trace, n_samples, delta, d_feat, err, st);
-  SampleSums hs;
-  uint32_t herr = 0;
-  std::memset(&hs, 0, sizeof(hs));
+  struct {
+    SampleSums sums;
+    uint32_t err;  // at sums + 1 on the device
+  } h;
+  std::memset(&h, 0, sizeof(h));
   if (s == TC_OK) {
-    e = cudaMemcpyAsync(&hs, sums, sizeof(hs), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = read_back(&h, sums, sizeof(h.sums) + sizeof(h.err), st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_sample_features");
   }
   if (trace) cudaFreeAsync(trace, st);
   if (sums) cudaFreeAsync(sums, st);
-  if (s == TC_OK && (hs.err | herr)) s = device_status(hs.err | herr, "tc_sample_features");
+  if (s == TC_OK && (h.sums.err | h.err)) s = device_status(h.sums.err | h.err, "tc_sample_features");
   return s;
 }
 
@@ -714,8 +746,7 @@ tc_status tc_mlp_grad_ex(const tc_mlp* mlp, const uint16_t* d_feat, const uint32
   }
   float hl = 0.f;
   if (s == TC_OK) {
-    e = cudaMemcpyAsync(&hl, loss, sizeof(float), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = read_back(&hl, loss, sizeof(float), st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_mlp_grad");
   }
   cudaFreeAsync(buf, st);
@@ -780,10 +811,9 @@ tc_status tc_mlp_train_ex(tc_mlp* mlp, const tc_graph* g, const tc_motif* motif,
   SampleSums hs;
   float first = 0.f, last = 0.f;
   if (s == TC_OK) {
-    e = cudaMemcpyAsync(&hs, sums, sizeof(hs), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&first, losses, sizeof(float), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&last, losses + steps - 1, sizeof(float), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = read_back(&hs, sums, sizeof(hs), st);
+    if (e == cudaSuccess) e = read_back(&first, losses, sizeof(float), st);
+    if (e == cudaSuccess) e = read_back(&last, losses + steps - 1, sizeof(float), st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_mlp_train");
   }
   for (void* p : {(void*)trace, (void*)rows, (void*)labels, (void*)losses, (void*)sums, vbuf})
@@ -839,10 +869,13 @@ tc_status tc_proposal_weights(const tc_mlp* mlp, const tc_graph* g, const tc_mot
   it.stop();
   uint32_t h_err = 0;
   if (s == TC_OK && h_Q) {
-    e = cudaMemcpyAsync(h_Q, d_qprefix + m, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    IndexHeader h;  // as in tc_path_weights
+    e = read_back(&h, d_qindex, sizeof(h), st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_proposal_weights");
+    if (s == TC_OK) {
+      *h_Q = h.W;
+      h_err = h.status;
+    }
   }
   cudaFreeAsync(scratch, st);
   if (s == TC_OK && h_err) s = device_status(h_err, "tc_proposal_weights");
@@ -876,9 +909,8 @@ tc_status tc_sample_estimate_q(const tc_graph* g, const tc_motif* motif, int64_t
   SampleSums hs;
   std::memset(&hs, 0, sizeof(hs));
   if (s == TC_OK) {
-    e = cudaMemcpyAsync(hb.data(), bins, 8 * nbins, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, sums, sizeof(hs), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = read_back(hb.data(), bins, 8 * nbins, st);
+    if (e == cudaSuccess) e = read_back(&hs, sums, sizeof(hs), st);
     if (e != cudaSuccess) s = cuda_status(e, "tc_sample_estimate_q");
   }
   if (bins) cudaFreeAsync(bins, st);

@@ -1054,9 +1054,8 @@ tc_status build_graph(int64_t n, int64_t m, const int32_t* d_src, const int32_t*
   }
   uint32_t h_err = 0;
   long long h_tmm[2];
-  TRY_C(cudaMemcpyAsync(&h_err, err, sizeof(h_err), cudaMemcpyDeviceToHost, st), "memcpy");
-  TRY_C(cudaMemcpyAsync(h_tmm, tmm, sizeof(h_tmm), cudaMemcpyDeviceToHost, st), "memcpy");
-  TRY_C(cudaStreamSynchronize(st), "sync");
+  TRY_C(read_back(&h_err, err, sizeof(h_err), st), "memcpy");
+  TRY_C(read_back(h_tmm, tmm, sizeof(h_tmm), st), "memcpy");
   if (h_err & kErrBadId) return done(set_error(TC_ERR_INVALID_ARG, "vertex id outside [0, n)"));
   g->tmin = M ? h_tmm[0] : 0;
   g->tmax = M ? h_tmm[1] : 0;
@@ -1186,8 +1185,7 @@ tc_status build_graph(int64_t n, int64_t m, const int32_t* d_src, const int32_t*
     TC_LAUNCHED(1);
     TRY_C(cudaGetLastError(), "k_pair_count");
     TRY_S(scan_u32(psums, psums, ptiles, st));
-    TRY_C(cudaMemcpyAsync(&P, psums + ptiles, sizeof(uint32_t), cudaMemcpyDeviceToHost, st), "memcpy");
-    TRY_C(cudaStreamSynchronize(st), "sync");
+    TRY_C(read_back(&P, psums + ptiles, sizeof(uint32_t), st), "memcpy");
   } else if (M) {
     k_gather_key<<<gr, 256, 0, st>>>(d_src, va, M, ka);
     TC_LAUNCHED(1);

@@ -193,6 +193,12 @@ inline cudaError_t pool_malloc(T** p, size_t bytes, cudaStream_t st) {
 tc_status cuda_status(cudaError_t e, const char* what);
 tc_status device_status(uint32_t bits, const char* what);
 
+// Copies `bytes` of device memory to host memory and waits for the stream.
+// Small results go through a pinned buffer of the calling thread (freed with
+// it): a copy to pageable memory takes the driver's staging path, about ten
+// microseconds of a short call.
+cudaError_t read_back(void* host, const void* device, size_t bytes, cudaStream_t st);
+
 #define TC_CUDA(call)                                         \
   do {                                                        \
     cudaError_t _e = (call);                                  \

@@ -1713,8 +1713,7 @@ float* mlp_grad_buffer(tc_mlp* M) { return M->grad; }
 
 tc_status mlp_check_error(const tc_mlp* M, cudaStream_t st, const char* what) {
   uint32_t bits = 0;
-  TC_CUDA(cudaMemcpyAsync(&bits, M->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-  TC_CUDA(cudaStreamSynchronize(st));
+  TC_CUDA(read_back(&bits, M->err, sizeof(uint32_t), st));
   if (!bits) return TC_OK;
   TC_CUDA(cudaMemsetAsync(M->err, 0, sizeof(uint32_t), st));
   return device_status(bits, what);
