@@ -72,6 +72,8 @@ struct tc_batch {
   unsigned blocks[2] = {0, 0};
   bool use_graph = true;
   cudaStream_t cap = nullptr;
+  cudaStream_t side = nullptr;                  // the orders, beside the weights
+  cudaEvent_t fork = nullptr, join = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};  // run start, sampling start, sampling end
@@ -98,6 +100,9 @@ void batch_free(tc_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   if (b->cap) cudaStreamDestroy(b->cap);
+  if (b->side) cudaStreamDestroy(b->side);
+  if (b->fork) cudaEventDestroy(b->fork);
+  if (b->join) cudaEventDestroy(b->join);
   for (cudaEvent_t e : b->ev)
     if (e) cudaEventDestroy(e);
   for (void* p : b->allocations) cudaFree(p);
@@ -124,22 +129,34 @@ tc_status upload_tiles(tc_batch* b) {
 }
 
 // Everything before the sampling launch: clear the sums, build each slot's
-// weights, prefix and index, and put each query's samples in key order.
+// weights, prefix and index, and put each query's samples in order.  An order
+// depends on the query's seed and ids alone, so the orders run on a stream of
+// the batch's own beside the weights (their kernels are bound by issue, the
+// weights' by latency): 72 queries on a 1e7-edge graph and eight small ones,
+// 14.9 ms a run, and 15.9 ms one after the other.
 tc_status enqueue_prologue(tc_batch* b, cudaStream_t st) {
   const size_t nq = b->queries.size(), ns = b->slots.size();
   TC_CUDA(cudaMemsetAsync(b->sums, 0, sizeof(SampleSums) * nq, st));
   TC_CUDA(cudaMemsetAsync(b->err, 0, sizeof(uint32_t) * ns, st));
-  for (size_t s = 0; s < ns; s++) {
+  TC_CUDA(cudaEventRecord(b->fork, st));
+  TC_CUDA(cudaStreamWaitEvent(b->side, b->fork, 0));
+  tc_status order = TC_OK;  // a failed launch must not leave the side stream unjoined
+  for (const Record& R : b->work) {
+    if (!R.order || order != TC_OK) continue;
+    const tc_query& q = b->queries[R.query].q;
+    order = order_samples(q.seed, q.sample_offset + R.base, R.count, 1, b->sort_scratch, R.order, b->side);
+  }
+  TC_CUDA(cudaEventRecord(b->join, b->side));
+  tc_status weights = TC_OK;
+  for (size_t s = 0; s < ns && weights == TC_OK; s++) {
     const Slot& S = b->slots[s];
     EdgeWin* win = (EdgeWin*)(S.index + kIndexHeaderBytes);
-    TC_TRY(launch_weights_scan(S.g, S.plan, S.delta, win, S.prefix, nullptr, b->scan_scratch, b->err + s, st));
-    TC_TRY(launch_guide(S.g, S.plan, S.delta, S.prefix, S.index, b->err + s, st));
+    weights = launch_weights_scan(S.g, S.plan, S.delta, win, S.prefix, nullptr, b->scan_scratch, b->err + s, st);
+    if (weights == TC_OK) weights = launch_guide(S.g, S.plan, S.delta, S.prefix, S.index, b->err + s, st);
   }
-  for (const Record& R : b->work) {
-    if (!R.order) continue;
-    const tc_query& q = b->queries[R.query].q;
-    TC_TRY(order_samples(q.seed, q.sample_offset + R.base, R.count, 1, b->sort_scratch, R.order, st));
-  }
+  TC_CUDA(cudaStreamWaitEvent(st, b->join, 0));
+  TC_TRY(order);
+  TC_TRY(weights);
   return TC_OK;
 }
 
@@ -320,6 +337,9 @@ tc_status create(const tc_query* hq, int64_t nq, const tc_batch_options* opts, c
   }
   TC_CUDA(cudaMemcpy(b->records, b->h_records.data(), b->h_records.size(), cudaMemcpyHostToDevice));
   for (cudaEvent_t& e : b->ev) TC_CUDA(cudaEventCreate(&e));
+  TC_CUDA(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
+  TC_CUDA(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+  TC_CUDA(cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming));
   // launch shape
   const int bs = opts ? opts->block_size : 0;
   const uint32_t tile = opts ? opts->tile : 0;

@@ -263,11 +263,6 @@ tc_status scan_u64_from_tile_sums(const uint64_t* in, uint64_t* out, uint64_t n,
 
 uint64_t scan_tile_size() { return kScanTile; }
 
-tc_status scan_u32_in_scratch(const uint32_t* in, uint32_t* out, uint64_t n, uint32_t* scratch,
-                              uint64_t scratch_words, cudaStream_t st) {
-  return scan_in_scratch<uint32_t>(in, out, n, true, nullptr, scratch, scratch_words, st);
-}
-
 // ---------------------------------------------------------------------------
 // Stable LSD radix sort of (uint32 key, uint32 value).
 

@@ -271,11 +271,6 @@ __device__ __forceinline__ bool bounded_draw_words(uint64_t seed, uint64_t s, ui
   return false;
 }
 
-__device__ __forceinline__ bool bounded_draw(uint64_t seed, uint64_t s, uint32_t draw, uint64_t range,
-                                             uint64_t* out) {
-  return bounded_draw_words(seed, s, draw, false, range, out);
-}
-
 __device__ __forceinline__ int64_t sat_add(int64_t a, int64_t d) {
   return (a > INT64_MAX - d) ? INT64_MAX : a + d;
 }
@@ -338,35 +333,6 @@ __device__ __forceinline__ uint32_t gallop(uint32_t s, uint32_t f, uint32_t a, T
   return lo;
 }
 
-// Window of x's list (alpha < 0: in-list, else out-list) around time t
-// (beta < 0: before, else after; strict or closed at t) as positions [lo, hi).
-// The two bounds are searched independently so that their loads overlap.
-// Compact: the list times are read from the 32-bit arrays (t - tmin).
-template <bool Compact>
-__device__ __forceinline__ void window_range(const OutEdge* __restrict__ out_e,
-                                             const uint32_t* __restrict__ out_off,
-                                             const InEdge* __restrict__ in_e,
-                                             const uint32_t* __restrict__ in_off,
-                                             const uint32_t* __restrict__ out_t32,
-                                             const uint32_t* __restrict__ in_t32, int64_t tmin, int alpha,
-                                             int beta, int closed, int32_t x, int64_t t, int64_t delta,
-                                             uint32_t* lo, uint32_t* hi) {
-  const bool in = alpha < 0;
-  const uint32_t a = __ldg((in ? in_off : out_off) + x), b = __ldg((in ? in_off : out_off) + x + 1);
-  const uint32_t* t32 = in ? in_t32 : out_t32;
-  auto tt = [&](uint32_t p) -> int64_t {
-    if (Compact) return (int64_t)__ldg(t32 + p) + tmin;
-    return in ? in_e[p].t : out_e[p].t;
-  };
-  if (beta < 0) {
-    *lo = search_time<true>(a, b, sat_sub(t, delta), tt);
-    *hi = closed ? search_time<false>(a, b, t, tt) : search_time<true>(a, b, t, tt);
-  } else {
-    *lo = closed ? search_time<true>(a, b, t, tt) : search_time<false>(a, b, t, tt);
-    *hi = search_time<false>(a, b, sat_add(t, delta), tt);
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Host-side launchers (defined in the .cu files).
 
@@ -375,9 +341,7 @@ __device__ __forceinline__ void window_range(const OutEdge* __restrict__ out_e,
 // not overlap unless in == out.
 tc_status scan_u64(const uint64_t* in, uint64_t* out, uint64_t n, uint32_t* d_err, cudaStream_t st);
 tc_status scan_u32(const uint32_t* in, uint32_t* out, uint64_t n, cudaStream_t st);
-uint64_t scan_u64_scratch_words(uint64_t n);  // also the element count for u32 scans
-tc_status scan_u32_in_scratch(const uint32_t* in, uint32_t* out, uint64_t n, uint32_t* scratch,
-                              uint64_t scratch_words, cudaStream_t st);
+uint64_t scan_u64_scratch_words(uint64_t n);
 tc_status scan_u64_in_scratch(const uint64_t* in, uint64_t* out, uint64_t n, bool write_total, uint32_t* d_err,
                               uint64_t* scratch, uint64_t scratch_words, cudaStream_t st);
 // The same scan when the kernel that wrote `in` also wrote the sums of its
