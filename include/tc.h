@@ -479,9 +479,9 @@ typedef struct {
 typedef struct tc_batch tc_batch;
 
 /* Validates the queries (as tc_sample_estimate would), allocates the batch's
- * memory and, when block_size or tile is 0, times every candidate
- * (block size 128/256/512 x tile 2048/8192/32768) on one full run and keeps
- * the fastest.  opts may be NULL (autotune, use_graph = 1).  Synchronises
+ * memory and, when block_size or tile is 0, times candidates (the block
+ * sizes 128, 256 and 512, then the tiles 2048, 8192 and 32768 at the fastest
+ * of them) on one full run each and keeps the fastest.  opts may be NULL (autotune, use_graph = 1).  Synchronises
  * stream.  Errors: TC_ERR_INVALID_ARG for a NULL or bad argument,
  * TC_ERR_UNSUPPORTED_MOTIF, TC_ERR_OOM, TC_ERR_CUDA. */
 tc_status tc_batch_create(const tc_query* h_queries, int64_t nq, const tc_batch_options* opts, void* stream,

@@ -198,48 +198,48 @@ tc_status enqueue_all(tc_batch* b, cudaStream_t st) {
   return enqueue_epilogue(b, st);
 }
 
-// Times the sampling launch for every (block size, tile) candidate on the
-// prepared batch and keeps the fastest; the prologue runs once before.
+// Times the sampling launch on the prepared batch (the prologue runs once
+// before), first for the block sizes at the tile in hand, then for the other
+// tiles at the fastest block size, and keeps the fastest: a full run each, and
+// the two choices hardly bear on one another.
 tc_status autotune(tc_batch* b, bool tune_bs, bool tune_tile, cudaStream_t st) {
   TC_TRY(enqueue_prologue(b, st));
   cudaEvent_t e0, e1;
   TC_CUDA(cudaEventCreate(&e0));
   TC_CUDA(cudaEventCreate(&e1));
-  tc_status s = TC_OK;
   float best = 0.0f;
   int best_bs = b->block_size;
   uint32_t best_tile = b->tile;
   bool first = true;
-  for (int bs : kBlockSizes) {
-    if (!tune_bs && bs != b->block_size) continue;
-    for (uint32_t tile : kTiles) {
-      if (!tune_tile && tile != b->tile) continue;
-      b->block_size = bs;
-      b->tile = tile;
-      s = upload_tiles(b);
-      for (int rep = 0; rep < (first ? 2 : 1) && s == TC_OK; rep++) {  // the first candidate warms the caches
-        cudaError_t e = cudaMemsetAsync(b->sums, 0, sizeof(SampleSums) * b->queries.size(), st);
-        if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-        if (e != cudaSuccess) s = cuda_status(e, "autotune");
-        if (s == TC_OK) s = enqueue_sampling(b, st);
-        if (s == TC_OK) {
-          e = cudaEventRecord(e1, st);
-          if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-          if (e != cudaSuccess) s = cuda_status(e, "autotune");
-        }
-      }
-      if (s != TC_OK) break;
-      float ms = 0.0f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (first || ms < best) {
-        best = ms;
-        best_bs = bs;
-        best_tile = tile;
-      }
-      first = false;
+  auto time_candidate = [&](int bs, uint32_t tile) -> tc_status {
+    b->block_size = bs;
+    b->tile = tile;
+    TC_TRY(upload_tiles(b));
+    for (int rep = 0; rep < (first ? 2 : 1); rep++) {  // the first candidate warms the caches
+      TC_CUDA(cudaMemsetAsync(b->sums, 0, sizeof(SampleSums) * b->queries.size(), st));
+      TC_CUDA(cudaEventRecord(e0, st));
+      TC_TRY(enqueue_sampling(b, st));
+      TC_CUDA(cudaEventRecord(e1, st));
+      TC_CUDA(cudaEventSynchronize(e1));
     }
-    if (s != TC_OK) break;
-  }
+    float ms = 0.0f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    if (first || ms < best) {
+      best = ms;
+      best_bs = bs;
+      best_tile = tile;
+    }
+    first = false;
+    return TC_OK;
+  };
+  tc_status s = time_candidate(b->block_size, b->tile);
+  const int bs0 = b->block_size;
+  const uint32_t tile0 = b->tile;
+  for (int bs : kBlockSizes)
+    if (s == TC_OK && tune_bs && bs != bs0) s = time_candidate(bs, tile0);
+  const int bs1 = best_bs;
+  for (uint32_t tile : kTiles)
+    if (s == TC_OK && tune_tile && tile != tile0) s = time_candidate(bs1, tile);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   TC_TRY(s);
@@ -346,7 +346,7 @@ tc_status create(const tc_query* hq, int64_t nq, const tc_batch_options* opts, c
   b->use_graph = opts ? opts->use_graph != 0 : true;
   if (bs && !sample_batch_blocks_per_sm(bs, true)) return set_error(TC_ERR_INVALID_ARG, "block_size must be 128, 256 or 512");
   if (tile && (tile % (bs ? bs : 512)) != 0) return set_error(TC_ERR_INVALID_ARG, "tile must be a multiple of block_size");
-  b->block_size = bs ? bs : 256;
+  b->block_size = bs ? bs : 512;
   b->tile = tile ? tile : 8192;
   TC_TRY(upload_tiles(b));
   if (!bs || !tile) TC_TRY(autotune(b, bs == 0, tile == 0, st));
