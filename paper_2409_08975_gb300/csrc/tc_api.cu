@@ -69,9 +69,16 @@ cudaError_t read_back(void* host, const void* device, size_t bytes, cudaStream_t
         t_pinned.p = nullptr;
       }
     }
-    if (!t_pinned.p && cudaHostAlloc(&t_pinned.p, kPinnedBytes, cudaHostAllocPortable) != cudaSuccess) {
-      cudaGetLastError();
-      t_pinned.p = nullptr;
+    if (!t_pinned.p) {
+      // Another thread may be capturing a stream in global mode, which an
+      // allocation outside the relaxed mode would disturb.
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      if (cudaHostAlloc(&t_pinned.p, kPinnedBytes, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        t_pinned.p = nullptr;
+      }
+      cudaThreadExchangeStreamCaptureMode(&mode);
     }
     if (t_pinned.p) to = t_pinned.p;
   }
