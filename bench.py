@@ -51,7 +51,7 @@ MOTIF_NAMES = {str(v): k for k, v in MOTIFS.items()}
 # pass over the default workload's list build and five steps: the launch list
 # summarised in profiles/launch_list_large_bench.md); valid while the kernel
 # is unchanged, null for workloads not captured
-SAMPLER_TRAFFIC_PER_SAMPLE = {("large", "c4"): 76.3}   # k_sample
+SAMPLER_TRAFFIC_PER_SAMPLE = {("large", "c4"): 25.7}   # k_sample
 WEIGHTS_TRAFFIC_PER_EDGE = {("large", "c4"): 89.9}     # k_weights_rw 74.1 + the scan of w 15.8
 UNIT = "samples/s"
 SECTOR = 32
@@ -702,19 +702,22 @@ def main():
 
     peak, peak_kind = load_peaks()
     checked_frac = r0["checked"] / max(r0["k"], 1)
-    # sampler algorithmic bytes per sample (sector model): guide entry, prefix
-    # entry, edge record and the end-edge entries (two for a 3-path anchor,
-    # one for a wedge): 5 or 4 sectors; a checked path adds the pair-list
-    # lookup (hash slot and pair-list times: 4 sectors)
+    # sectors a sample touches (model): guide entry, prefix entry, edge record
+    # and the end-edge entries (two for a 3-path anchor, one for a wedge): 5 or
+    # 4 sectors; a checked path adds the pair-list lookup (hash slot and
+    # pair-list times: 4 sectors).  Ordered samples share them through L1 and
+    # L2, so the fraction of HBM is taken from the measured DRAM bytes where
+    # they are known.
     ends = sum(1 for a in (alpha1, alpha3) if a != 0)
     bytes_per_sample = SECTOR * (3 + ends + 4 * checked_frac)
-    achieved = bytes_per_sample * k / (ph["sample"] / 1e3) / 1e9
     key = (cfg["name"], MOTIF_NAMES.get(str([tuple(e) for e in cfg["motif"]])))
     tps = SAMPLER_TRAFFIC_PER_SAMPLE.get(key)
+    achieved = (tps or bytes_per_sample) * k / (ph["sample"] / 1e3) / 1e9
     roofline = {"bound": "hbm", "kernel": "k_sample (sampler with CheckMotif / ListCount, Alg. 2-4)",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": tps * k if tps else None, "peak_kind": peak_kind,
-                "limiter": "latency of dependent random loads (long-scoreboard stalls in ncu)",
+                "achieved_from": "measured DRAM bytes" if tps else "sector model",
+                "limiter": "latency of dependent random loads and issue at 48 warps per SM (ncu)",
                 "bytes_per_sample": bytes_per_sample, "kernel_ms": ph["sample"],
                 "dram_bytes_per_sample": tps,
                 "dram_frac": (tps * k / (ph["sample"] / 1e3) / 1e9 / peak) if tps else None}

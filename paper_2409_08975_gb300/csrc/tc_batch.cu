@@ -2,7 +2,7 @@
 // answered by one fixed launch sequence.  Weights, prefix and index are
 // built once per distinct (graph, anchor class, window kind, delta) -- the
 // weights of Claim 1 depend on nothing else -- every query's samples are put
-// in key order, and one persistent launch samples all queries (Alg. 2-5 per
+// in draw order, and one persistent launch samples all queries (Alg. 2-5 per
 // query).  The sequence allocates nothing, so it can be captured once into
 // a CUDA graph and replayed.
 #include <cuda_runtime.h>

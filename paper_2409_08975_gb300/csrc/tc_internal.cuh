@@ -457,7 +457,7 @@ tc_status order_samples(uint64_t seed, uint64_t first, uint64_t count, uint32_t 
                         cudaStream_t st);
 
 // Batched sampling: each record is the arguments of one query's samples
-// [chunk_base, chunk_base + count) (one chunk of them, in key order, or all
+// [chunk_base, chunk_base + count) (one chunk of them, in draw order, or all
 // of them in id order), kBatchQueryBytes bytes in device memory, written on
 // the host by batch_query_record; its sums are added to *sums.  The records'
 // work items (groups of buckets holding about `tile` samples, or tiles of
