@@ -419,12 +419,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t* _
 tc_status radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint64_t n, int bit0,
                            int bit1, cudaStream_t st) {
   if (n <= 1 || bit1 <= bit0) return TC_OK;
-  static bool attr = false;
-  if (!attr) {
-    TC_CUDA(cudaFuncSetAttribute(k_sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(uint32_t) * sort_scatter_words(kMaxRadix))));
-    attr = true;
-  }
+  TC_CUDA(allow_shared(k_sort_scatter, sizeof(uint32_t) * sort_scatter_words(kMaxRadix)));
   const int total = bit1 - bit0;
   const int passes = (total + kMaxDigitBits - 1) / kMaxDigitBits;
   const int width = (total + passes - 1) / passes;
@@ -640,12 +635,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_rec_scatter(const __grid_con
 // the result (with no bits the records are copied, or stay where they are).
 static tc_status rec_sort(RecSource R, uint64_t n, int word, int bits, uint4* a, uint4* b, uint32_t* hist,
                           const uint4** sorted, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    TC_CUDA(cudaFuncSetAttribute(k_rec_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)rec_scatter_bytes(kMaxRadix)));
-    attr = true;
-  }
+  TC_CUDA(allow_shared(k_rec_scatter, rec_scatter_bytes(kMaxRadix)));
   const uint32_t tiles = (uint32_t)((n + kRecTile - 1) / kRecTile);
   const int passes = bits > 0 ? (bits + kMaxDigitBits - 1) / kMaxDigitBits : 1;  // no bits: one pass of one digit
   const int width = (bits + passes - 1) / passes;

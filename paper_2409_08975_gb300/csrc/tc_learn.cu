@@ -1621,12 +1621,7 @@ template <bool Proposal>
 static tc_status launch_umma(const tc_mlp* M, const uint16_t* feat, const uint32_t* rows, uint64_t n, float* logits,
                              const uint64_t* prefix, float eps, float scale, uint16_t* h, uint64_t* q,
                              uint64_t* tile_sums, uint32_t* hrange, uint32_t* d_err, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    TC_CUDA(cudaFuncSetAttribute(k_mlp_umma<Proposal>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kUmmaSmemBytes));
-    attr = true;
-  }
+  TC_CUDA(allow_shared(k_mlp_umma<Proposal>, kUmmaSmemBytes));
   // umma_blocks_per_sm blocks per SM: what the launch bounds' registers and the
   // shared memory allow (their TMEM, 64 columns each, fits an SM's 512)
   const uint64_t T = Proposal ? (n + kUmmaTile - 1) / kUmmaTile : (n + kUmmaM - 1) / kUmmaM;
@@ -1660,11 +1655,7 @@ tc_status launch_mlp_forward(const tc_mlp* M, const uint16_t* feat, const uint32
 static tc_status launch_grad(const tc_mlp* M, const uint16_t* feat, const uint32_t* rows, const float* labels,
                              uint64_t n, float* grad, float* loss_sum, const float* z, const VarianceSums* V, float eps,
                              cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    TC_CUDA(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainShared)));
-    attr = true;
-  }
+  TC_CUDA(allow_shared(k_mlp_grad, sizeof(TrainShared)));
   static_assert(2 * (sizeof(TrainShared) + 1024) <= 227 * 1024, "two gradient blocks per SM");
   const uint64_t tiles = (n + kTrainRows - 1) / kTrainRows, fit = (uint64_t)num_sms() * 2;
   k_mlp_grad<<<(unsigned)(tiles < fit ? tiles : fit), 32 * kTrainWarps, sizeof(TrainShared), st>>>(
@@ -1761,13 +1752,8 @@ tc_status launch_proposal_scan(const tc_mlp* M, const uint16_t* feat, const uint
     TC_TRY(launch_umma<true>(M, feat, nullptr, m, nullptr, prefix, eps, scale, h, q, sums, hrange, d_err, st));
     return scan_u64_from_tile_sums(q, qprefix, m, sums, d_err, scan_scratch, scan_u64_scratch_words(T) + 1, st);
   }
-  static int bps = 0;
-  if (!bps) {
-    TC_CUDA(cudaFuncSetAttribute(k_proposal, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPDynSmem));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_proposal, kPThreads, kPDynSmem);
-    if (bps <= 0) bps = 1;
-  }
-  uint64_t blocks = (uint64_t)num_sms() * bps;
+  TC_CUDA(allow_shared(k_proposal, kPDynSmem));
+  uint64_t blocks = (uint64_t)num_sms() * blocks_per_sm(k_proposal, kPThreads, kPDynSmem);
   if (blocks > T) blocks = T;
   k_proposal<<<(unsigned)blocks, kPThreads, kPDynSmem, st>>>(M->params, reinterpret_cast<const __nv_bfloat16*>(feat),
                                                              prefix, m, eps, scale, h, q, sums, hrange, d_err);

@@ -1252,12 +1252,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_second(const uint32_t* 
 // of order_scratch_bytes bytes (no allocation).
 tc_status order_samples(uint64_t seed, uint64_t first, uint64_t count, uint32_t wave, void* scratch, void* order,
                         cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    TC_CUDA(cudaFuncSetAttribute(k_order_second, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(OrderSecondShared)));
-    attr = true;
-  }
+  TC_CUDA(allow_shared(k_order_second, sizeof(OrderSecondShared)));
   const OrderPlan L = order_plan(count, wave);
   uint32_t* head = (uint32_t*)order;
   uint32_t* cursor1 = head + kOrderHeadWords;
@@ -1586,16 +1581,8 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
   auto kernel = trace ? (compact ? k_sample<true, true> : k_sample<true, false>)
                       : (compact ? k_sample<false, true> : k_sample<false, false>);
   constexpr size_t kTileBytes = sizeof(TileShared<kSampleThreads>);
-  static int blocks_per_sm[4] = {0, 0, 0, 0};
-  const int ti = (trace ? 2 : 0) + (compact ? 1 : 0);
-  if (!blocks_per_sm[ti]) {
-    int b = 0;
-    TC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kTileBytes + kSmemBinBytes)));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kSampleThreads, kTileBytes + kSmemBinBytes);
-    blocks_per_sm[ti] = b > 0 ? b : 1;
-  }
-  const uint64_t max_blocks = (uint64_t)num_sms() * blocks_per_sm[ti];
+  TC_CUDA(allow_shared(kernel, kTileBytes + kSmemBinBytes));
+  const uint64_t max_blocks = (uint64_t)num_sms() * blocks_per_sm(kernel, kSampleThreads, kTileBytes + kSmemBinBytes);
   auto run = [&](const OrderView& ord, uint64_t base, uint64_t count) -> tc_status {
     A.ord = ord;
     A.chunk_base = base;
@@ -1670,10 +1657,8 @@ tc_status launch_path_sum(const tc_graph* g, const Plan& plan, int64_t delta, co
   A.delta = delta;
   A.graph_id = g->id;
   A.sums = d_sums;
-  int bps = 0;
   auto kernel = A.pair_t32 ? k_path_sum<true> : k_path_sum<false>;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, 256, 0);
-  uint64_t blocks = (uint64_t)num_sms() * (bps > 0 ? bps : 1);
+  uint64_t blocks = (uint64_t)num_sms() * blocks_per_sm(kernel, 256, 0);
   const uint64_t need = (W + 255) / 256;
   if (need < blocks) blocks = need ? need : 1;
   // as many paths for every warp: runs of at most kPathRun, as many of them
@@ -1838,15 +1823,8 @@ __global__ void __launch_bounds__(BS, (512 * TC_SAMPLE_MIN_BLOCKS) / BS)
 
 template <int BS, bool Compact>
 static int batch_blocks_per_sm() {
-  static int cached = 0;
-  if (!cached) {
-    int b = 0;
-    cudaFuncSetAttribute(k_sample_batch<BS, Compact>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(TileShared<BS>));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample_batch<BS, Compact>, BS, sizeof(TileShared<BS>));
-    cached = b > 0 ? b : 1;
-  }
-  return cached;
+  static_assert(sizeof(TileShared<BS>) + 1024 <= 48 << 10, "with the static part: more has to be allowed first");
+  return blocks_per_sm(k_sample_batch<BS, Compact>, BS, sizeof(TileShared<BS>));
 }
 
 int sample_batch_blocks_per_sm(int bs, bool compact) {
