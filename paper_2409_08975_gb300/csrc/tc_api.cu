@@ -1,5 +1,6 @@
 // C ABI of the library (include/tc.h): argument checks, the motif compiler,
 // object lifetime, error reporting and the host arithmetic of the estimate.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -48,43 +49,92 @@ cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+bool current_context_id(unsigned long long* id) {
+  // driver entry points reached through the runtime, so the library does not link libcuda
+  struct Driver {
+    CUresult (*get_current)(CUcontext*) = nullptr;
+    CUresult (*get_id)(CUcontext, unsigned long long*) = nullptr;
+    static void* entry(const char* name) {
+      void* f = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &q);
+      return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? f : nullptr;
+    }
+    Driver() {
+      get_current = (decltype(get_current))entry("cuCtxGetCurrent");
+      get_id = (decltype(get_id))entry("cuCtxGetId");
+    }
+  };
+  static const Driver driver;
+  CUcontext ctx = nullptr;
+  return driver.get_current && driver.get_id && driver.get_current(&ctx) == CUDA_SUCCESS && ctx &&
+         driver.get_id(ctx, id) == CUDA_SUCCESS;
+}
+
 namespace {
+
+// Pinned buffers of read_back, taken for one copy and given back after it: at
+// most kPinnedSlots in the process.  None is freed: a release waits for the
+// device and ends another thread's stream capture (in the global mode) in an
+// error.  A buffer serves the context that it was allocated in only, by the
+// context's id, which is never given out twice: a device reset takes its
+// buffers with it, and their addresses may then belong to someone else.
 constexpr size_t kPinnedBytes = 128 << 10;
-struct PinnedBuffer {
-  void* p = nullptr;
-  ~PinnedBuffer() {
-    if (p) cudaFreeHost(p);
-  }
+constexpr int kPinnedSlots = 16;
+struct PinnedSlot {
+  void* p;
+  unsigned long long ctx;
+  bool busy;
 };
-thread_local PinnedBuffer t_pinned;
+std::mutex g_pinned_mu;
+PinnedSlot g_pinned[kPinnedSlots];
+
+// NULL when no buffer can be had.
+PinnedSlot* take_pinned() {
+  unsigned long long ctx = 0;
+  if (!current_context_id(&ctx)) return nullptr;
+  PinnedSlot* s = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_pinned_mu);
+    for (PinnedSlot& x : g_pinned) {
+      if (x.busy) continue;
+      if (x.p && x.ctx == ctx) {
+        x.busy = true;
+        return &x;
+      }
+      if (!x.p && !s) s = &x;
+    }
+    if (!s) return nullptr;
+    s->busy = true;
+  }
+  // Another thread may be capturing a stream in the global mode, which an
+  // allocation outside the relaxed mode would disturb.
+  void* p = nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (cudaHostAlloc(&p, kPinnedBytes, cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  std::lock_guard<std::mutex> lock(g_pinned_mu);
+  s->p = p;
+  s->ctx = ctx;
+  s->busy = p != nullptr;
+  return p ? s : nullptr;
+}
+
 }  // namespace
 
 cudaError_t read_back(void* host, const void* device, size_t bytes, cudaStream_t st) {
-  void* to = host;
-  if (bytes <= kPinnedBytes) {
-    if (t_pinned.p) {  // a device reset takes the buffer with it
-      cudaPointerAttributes a;
-      if (cudaPointerGetAttributes(&a, t_pinned.p) != cudaSuccess || a.type != cudaMemoryTypeHost) {
-        cudaGetLastError();
-        t_pinned.p = nullptr;
-      }
-    }
-    if (!t_pinned.p) {
-      // Another thread may be capturing a stream in global mode, which an
-      // allocation outside the relaxed mode would disturb.
-      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-      cudaThreadExchangeStreamCaptureMode(&mode);
-      if (cudaHostAlloc(&t_pinned.p, kPinnedBytes, cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        t_pinned.p = nullptr;
-      }
-      cudaThreadExchangeStreamCaptureMode(&mode);
-    }
-    if (t_pinned.p) to = t_pinned.p;
-  }
-  cudaError_t e = cudaMemcpyAsync(to, device, bytes, cudaMemcpyDeviceToHost, st);
+  PinnedSlot* s = bytes <= kPinnedBytes ? take_pinned() : nullptr;
+  cudaError_t e = cudaMemcpyAsync(s ? s->p : host, device, bytes, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && to != host) std::memcpy(host, to, bytes);
+  if (s) {
+    if (e == cudaSuccess) std::memcpy(host, s->p, bytes);
+    std::lock_guard<std::mutex> lock(g_pinned_mu);
+    s->busy = false;
+  }
   return e;
 }
 

