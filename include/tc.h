@@ -205,6 +205,11 @@ tc_status tc_path_weights(const tc_graph* g, const tc_motif* motif, int64_t delt
  *                      motif and delta (checked on the device)
  *   h_out     receives the sums and the estimate (synchronises the stream)
  * Ranges [offset, offset + k) of one seed can be merged by adding the sums.
+ * Scratch: calls of 2^19 samples or more order them in chunks, about 11 bytes
+ * a sample of a chunk, from the library's pool, which keeps its memory for
+ * later calls.  A chunk has up to 2^28 samples (2.9 GB), and up to 2^30 (11
+ * GB) on graphs whose build took that much scratch from the same pool (52
+ * bytes an edge).
  * Errors: TC_ERR_INVALID_ARG, TC_ERR_OVERFLOW, TC_ERR_RNG_EXHAUSTED,
  * TC_ERR_CUDA.
  */
@@ -459,8 +464,10 @@ tc_status tc_sample_estimate_q(const tc_graph* g, const tc_motif* motif, int64_t
  *
  * Graphs are borrowed: they must outlive the batch.  The batch owns device
  * memory for each distinct weights key (prefix and index, 8 (m + 1) plus
- * tc_sample_index_bytes) and about 4.6 k bytes of sample order per query
- * with k >= 65536; k may be at most 2^40.
+ * tc_sample_index_bytes), about 4.6 k bytes of sample order per query
+ * with k >= 65536, and one scratch for ordering them of about 6 bytes a
+ * sample of the largest query with k beyond 4e6 (of at most 2^28 samples:
+ * 1.6 GB); k may be at most 2^40.
  */
 typedef struct {
   const tc_graph* graph;

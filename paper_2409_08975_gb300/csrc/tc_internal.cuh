@@ -468,7 +468,10 @@ struct OrderView {
 constexpr uint64_t kOrderedMinSamples = 1ull << 19;
 constexpr uint64_t kBatchOrderedMinSamples = 1ull << 16;
 constexpr uint64_t kChunkSamples = 1ull << 30;
-constexpr uint64_t kSmallChunkSamples = 1ull << 28;  // of a batch, and where memory is short
+constexpr uint64_t kSmallChunkSamples = 1ull << 28;  // of a batch, and see sample_chunk
+// Scratch that the build of a graph takes for each edge, beside its lists:
+// three records and the canonical position (more with 64-bit times).
+constexpr uint64_t kBuildScratchBytes = 3 * 16 + 4;
 size_t order_bytes(uint64_t count, uint32_t wave);
 size_t order_scratch_bytes(uint64_t count, uint32_t wave);
 OrderView order_view(uint64_t count, uint32_t wave, void* order);

@@ -1023,9 +1023,8 @@ __device__ __forceinline__ void sample_one(const SamplerArgs& A, const Plan& P, 
 // their histograms and scans took 12.4 ms and the sampler on that order 52.6
 // ms.  A sampler on the order by 20, 24 or 32 bits of the draw, otherwise
 // unchanged, took 43.5, 38.7 and 39.0 ms: beyond 24 bits (the bucket and its
-// bins here) nothing more is gained.  Chunks are as large as memory allows (up
-// to 2^30): each chunk reads the graph once from DRAM, and in chunks of 2^28
-// the sampler took 28.9 ms.
+// bins here) nothing more is gained.  Each chunk reads the graph once from
+// DRAM: in chunks of 2^28 the sampler took 28.9 ms (sample_chunk).
 constexpr int kOrderThreads = 512;
 constexpr int kOrderItems = 16;
 constexpr int kOrderTile = kOrderThreads * kOrderItems;  // 8192
@@ -1537,6 +1536,31 @@ float last_phase_ms(int phase) {
 
 float last_sampler_ms() { return last_phase_ms(TC_PHASE_SAMPLE); }
 
+// Scratch and order of a call of k samples in chunks of `chunk`: the last chunk
+// is smaller than the others, but its order may hold more rounding.
+static void chunk_bytes(uint64_t k, uint64_t chunk, uint32_t wave, size_t* scratch, size_t* order) {
+  const uint64_t tail = k % chunk;
+  *scratch = std::max(order_scratch_bytes(chunk, wave), tail ? order_scratch_bytes(tail, wave) : (size_t)0);
+  *order = std::max(order_bytes(chunk, wave), tail ? order_bytes(tail, wave) : (size_t)0);
+}
+
+// Samples a chunk, about 11 bytes each: 2^28 (2.9 GB), or up to 2^30 on graphs
+// whose own build took as much scratch.  The pool keeps what it has taken, so
+// such a chunk needs no more memory than the process has lent it before, and
+// the graphs that gain from reading them once are large (300M edges, 1e9
+// samples: 41.1 ms, in chunks of 2^28 45.6 ms).  Growing the pool by 11 GB for
+// a call and trimming it afterwards would take 9 and 15 ms.
+static uint64_t sample_chunk(uint64_t k, uint64_t m, uint32_t wave) {
+  uint64_t chunk = std::min(k, kChunkSamples);
+  while (chunk > kSmallChunkSamples) {
+    size_t scratch, order;
+    chunk_bytes(k, chunk, wave, &scratch, &order);
+    if (scratch + order <= kBuildScratchBytes * m) break;
+    chunk = std::max(chunk / 2, kSmallChunkSamples);
+  }
+  return chunk;
+}
+
 tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, const uint64_t* prefix,
                          const void* index, uint64_t k, uint64_t seed, uint64_t offset, uint64_t* trace,
                          SampleSums* d_sums, cudaStream_t st, const void* qindex, const uint16_t* h,
@@ -1603,17 +1627,15 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
     timer.stop();
     return s;
   }
-  // samples in chunks, each with an order of its own (about 11 bytes a sample;
-  // smaller chunks when the memory for a large one is not there)
+  // samples in chunks, each with an order of its own (smaller chunks also when
+  // the memory for a large one is not there)
   const uint32_t wave = (uint32_t)max_blocks;
-  uint64_t chunk = std::min(k, kChunkSamples);
+  uint64_t chunk = sample_chunk(k, m, wave);
   size_t scratch = 0;
   char* buf = nullptr;
   for (;;) {
-    // the last chunk is smaller than the others, but its order may hold more rounding
-    const uint64_t tail = k % chunk;
-    scratch = std::max(order_scratch_bytes(chunk, wave), tail ? order_scratch_bytes(tail, wave) : (size_t)0);
-    const size_t obytes = std::max(order_bytes(chunk, wave), tail ? order_bytes(tail, wave) : (size_t)0);
+    size_t obytes = 0;
+    chunk_bytes(k, chunk, wave, &scratch, &obytes);
     const cudaError_t e = pool_malloc(&buf, scratch + obytes, st);
     if (e == cudaSuccess) break;
     if (e != cudaErrorMemoryAllocation || chunk <= kSmallChunkSamples) return cuda_status(e, "pool_malloc(order)");

@@ -153,3 +153,46 @@ def test_read_back_buffers_are_shared_and_bounded(fake):
         L.fake_reset()
         call()
     assert L.fake_pinned_taken() <= 16 and L.fake_pinned_given() == given and not failed
+
+
+def test_large_calls_do_not_grow_the_pool_beyond_a_small_chunk(fake):
+    from paper_2409_08975_gb300 import tc
+    L = fake
+    L.fake_reserved.restype, L.fake_limit.argtypes = ctypes.c_size_t, [ctypes.c_size_t]
+    L.cudaSetDevice(1)
+    g = make_graph(L, [1, 2, 3])
+    mot, est = ctypes.byref(tc.make_motif(C4)), tc.tc_estimate()
+    prefix, p = buffer(8 * 4)
+    ib = ctypes.c_size_t()
+    assert L.tc_sample_index_bytes(g, ctypes.byref(ib)) == 0
+    index, ix = buffer(ib.value)
+    k = (1 << 30) + 600_001  # a ragged last chunk
+
+    def chunks(g, ix):
+        before = L.fake_launches(1, b"k_order_first")
+        status = L.tc_sample_estimate(g, mot, 10, p, ix, k, 1, 0, ctypes.byref(est), None)
+        return status, L.fake_launches(1, b"k_order_first") - before
+
+    before = L.fake_reserved()
+    L.fake_limit(2 << 30)  # not even a small chunk: an error, as ever
+    assert chunks(g, ix) == (2, 0)
+    L.fake_limit(ctypes.c_size_t(-1).value)
+    for _ in range(2):
+        assert chunks(g, ix) == (0, 5)
+        assert L.fake_reserved() <= before + (3 << 30)
+    # on a large graph the chunks take the memory that its build has left, and no more
+    for m, expected in ((120_000_000, 3), (240_000_000, 2)):
+        s, t = np.zeros(m, np.int32), np.zeros(m, np.int64)
+        big = ctypes.c_void_p()
+        assert L.tc_build_temporal_csr(m, m, s.ctypes.data, s.ctypes.data, t.ctypes.data, None, ctypes.byref(big)) == 0
+        assert L.tc_sample_index_bytes(big, ctypes.byref(ib)) == 0
+        index, ix = buffer(ib.value)
+        held = L.fake_reserved()
+        assert chunks(big, ix) == (0, expected)
+        assert L.fake_reserved() == held
+        if m > 200_000_000:  # memory is short after all: smaller chunks
+            L.fake_limit(held - 52 * m + (9 << 30))  # of the build's scratch, 9 GB are left
+            assert chunks(big, ix) == (0, 3)
+            L.fake_limit(ctypes.c_size_t(-1).value)
+        L.tc_graph_destroy(big)
+    L.tc_graph_destroy(g)
