@@ -195,9 +195,6 @@ static tc_status scan_rec(const T* in, T* out, uint64_t n, bool write_total, uin
   return s;
 }
 
-tc_status scan_u64(const uint64_t* in, uint64_t* out, uint64_t n, uint32_t* d_err, cudaStream_t st) {
-  return scan_rec<uint64_t>(in, out, n, true, d_err, st);
-}
 tc_status scan_u32(const uint32_t* in, uint32_t* out, uint64_t n, cudaStream_t st) {
   return scan_rec<uint32_t>(in, out, n, true, nullptr, st);
 }

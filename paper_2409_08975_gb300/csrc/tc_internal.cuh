@@ -355,10 +355,9 @@ __device__ __forceinline__ uint32_t gallop(uint32_t s, uint32_t f, uint32_t a, T
 // ---------------------------------------------------------------------------
 // Host-side launchers (defined in the .cu files).
 
-// Exclusive scans.  scan_u64 writes out[0..n] (out[n] = total) and sets
-// kErrOverflow in *d_err when the total exceeds 64 bits.  in and out must
-// not overlap unless in == out.
-tc_status scan_u64(const uint64_t* in, uint64_t* out, uint64_t n, uint32_t* d_err, cudaStream_t st);
+// Exclusive scans: out[0..n] (out[n] = total, where write_total); those of 64
+// bits set kErrOverflow in *d_err when the total exceeds 64 bits.  in and out
+// must not overlap unless in == out.
 tc_status scan_u32(const uint32_t* in, uint32_t* out, uint64_t n, cudaStream_t st);
 uint64_t scan_u64_scratch_words(uint64_t n);
 tc_status scan_u64_in_scratch(const uint64_t* in, uint64_t* out, uint64_t n, bool write_total, uint32_t* d_err,
@@ -463,7 +462,7 @@ struct OrderView {
   uint32_t* head;
   const uint32_t* sizes;
   const uint32_t* ids;
-  uint32_t nb, nb1, nb2, room;
+  uint32_t nb, room;
 };
 constexpr uint64_t kOrderedMinSamples = 1ull << 19;
 constexpr uint64_t kBatchOrderedMinSamples = 1ull << 16;

@@ -35,16 +35,6 @@ namespace tc {
 // A wedge anchor (3-vertex motif) has one window, at u or at v; the other
 // side is the dummy [0, 1), so w_e is the size of that window.
 
-// Window searches on the 32-bit time arrays when the graph has them.
-#ifndef TC_COMPACT_TIMES
-#define TC_COMPACT_TIMES 1
-#endif
-
-// Pair-list searches of the sampler on the 32-bit times when the graph has them.
-#ifndef TC_COMPACT_PAIRS
-#define TC_COMPACT_PAIRS 1
-#endif
-
 // Resident blocks per SM the weights kernel is compiled for (caps its registers).
 #ifndef TC_WEIGHTS_MIN_BLOCKS
 #define TC_WEIGHTS_MIN_BLOCKS 8
@@ -81,8 +71,7 @@ struct WeightsArgs {
   const uint2* x_in;  // anchors and their range words
   const uint2* x_out;
   const uint2* out2in;
-  // range word of the edge in u's out-list
-  const uint32_t* r_self;
+  const uint32_t* r_self;  // range word of the edge in u's out-list
   int64_t tmin;
   uint64_t m;
   int64_t delta;
@@ -93,23 +82,22 @@ struct WeightsArgs {
   uint32_t* err;
 };
 
-// Window of side alpha (< 0: the vertex's in-list, > 0: its out-list) of
-// canonical edge i = (x, ., t), searched from anchor a.
-template <bool Compact>
+// Graphs without 32-bit list times.  Window of side alpha (< 0: the vertex's
+// in-list, > 0: its out-list) of canonical edge i = (x, ., t), searched from
+// anchor a.
 __device__ __forceinline__ void side_window(const WeightsArgs& A, int alpha, int beta, int32_t x, uint32_t a,
                                             int64_t t, uint32_t* lo, uint32_t* hi) {
   if (alpha < 0) {
-    auto tt = [&](uint32_t p) -> int64_t { return Compact ? (int64_t)__ldg(A.in_t32 + p) + A.tmin : A.in_e[p].t; };
+    auto tt = [&](uint32_t p) -> int64_t { return A.in_e[p].t; };
     window_from(__ldg(A.in_off + x), __ldg(A.in_off + x + 1), a, beta, A.closed, t, A.delta, tt, lo, hi);
   } else {
-    auto tt = [&](uint32_t p) -> int64_t { return Compact ? (int64_t)__ldg(A.out_t32 + p) + A.tmin : A.out_e[p].t; };
+    auto tt = [&](uint32_t p) -> int64_t { return A.out_e[p].t; };
     window_from(__ldg(A.out_off + x), __ldg(A.out_off + x + 1), a, beta, A.closed, t, A.delta, tt, lo, hi);
   }
 }
 
 // Block b takes tile b: the windows and w of its kWTile edges (coalesced:
 // edge b kWTile + j 256 + thread), and the tile's sum of w.
-template <bool Compact>
 __global__ void __launch_bounds__(kWThreads, TC_WEIGHTS_MIN_BLOCKS) k_weights(const __grid_constant__ WeightsArgs A) {
   __shared__ unsigned long long s_warp[kWThreads / 32];
   __shared__ uint32_t s_ovf;
@@ -127,11 +115,10 @@ __global__ void __launch_bounds__(kWThreads, TC_WEIGHTS_MIN_BLOCKS) k_weights(co
     // anchors: u's in-list (x_in) or the edge itself in u's out-list; the
     // edge itself in v's in-list (out2in) or v's out-list (x_out)
     if (A.alpha1 != 0)
-      side_window<Compact>(A, A.alpha1, A.beta1, e.src, A.alpha1 < 0 ? __ldg(&A.x_in[i].x) : (uint32_t)i, e.t, &lo1,
-                           &hi1);
+      side_window(A, A.alpha1, A.beta1, e.src, A.alpha1 < 0 ? __ldg(&A.x_in[i].x) : (uint32_t)i, e.t, &lo1, &hi1);
     if (A.alpha3 != 0)
-      side_window<Compact>(A, A.alpha3, A.beta3, e.dst, A.alpha3 < 0 ? __ldg(&A.out2in[i].x) : __ldg(&A.x_out[i].x), e.t,
-                           &lo3, &hi3);
+      side_window(A, A.alpha3, A.beta3, e.dst, A.alpha3 < 0 ? __ldg(&A.out2in[i].x) : __ldg(&A.x_out[i].x), e.t, &lo3,
+                  &hi3);
     EdgeWin r;
     r.lo1 = lo1;
     r.d1 = hi1 - lo1;
@@ -297,11 +284,10 @@ tc_status launch_weights_scan(const tc_graph* g, const Plan& plan, int64_t delta
   A.w = wbuf;
   A.tile_sums = sums;
   A.err = d_err;
-  const bool compact = TC_COMPACT_TIMES && g->out_t32 && g->in_t32;
-  if (compact)
+  if (g->out_t32)  // 32-bit list times
     k_weights_rw<<<(unsigned)T, kWThreads, 0, st>>>(A);
   else
-    k_weights<false><<<(unsigned)T, kWThreads, 0, st>>>(A);
+    k_weights<<<(unsigned)T, kWThreads, 0, st>>>(A);
   TC_LAUNCHED(1);
   TC_CUDA(cudaGetLastError());
   return scan_u64_from_tile_sums(wbuf, prefix, m, sums, d_err, scan_scratch, scan_u64_scratch_words(T) + 1, st);
@@ -449,7 +435,7 @@ struct SamplerArgs {
   const IndexHeader* hdr;
   const EdgeWin* win;
   const uint32_t* guide;
-  uint64_t k, seed, offset;
+  uint64_t seed, offset;
   uint64_t chunk_base;    // index of the chunk's first sample within the call
   uint64_t count;         // samples in the chunk
   OrderView ord;          // the chunk's samples by buckets of their draws (nb = 0: in id order)
@@ -483,7 +469,6 @@ struct SampleTime {
     const uint64_t x = (uint64_t)first + (uint64_t)A.delta;  // delta < 2^63
     return x > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)x;
   }
-  static __device__ __forceinline__ int64_t absolute(const SamplerArgs& A, T t) { return (int64_t)t + A.tmin; }
 };
 template <>
 struct SampleTime<false> {
@@ -494,7 +479,6 @@ struct SampleTime<false> {
     return (uint64_t)last - (uint64_t)first > (uint64_t)A.delta;
   }
   static __device__ __forceinline__ T end(const SamplerArgs& A, T first) { return sat_add(first, A.delta); }
-  static __device__ __forceinline__ int64_t absolute(const SamplerArgs&, T t) { return t; }
 };
 
 // Positions [*s, *e) of the pair list L_{x,y} (empty when x never sends to
@@ -1008,7 +992,7 @@ __device__ __forceinline__ void sample_one(const SamplerArgs& A, const Plan& P, 
 // is uniform over 2^32.  Each chunk's ids are partitioned into nb = nb1 nb2
 // buckets of equal width of y (two passes of nb1 and nb2 buckets, one pass
 // for few buckets), and the sampler's block orders one bucket at a time in
-// shared memory (sample_buckets).
+// shared memory (sample_bucket).
 //
 // The bucket sizes are binomial, so every bucket gets a fixed room of its
 // mean plus eight standard deviations: a tile reserves its run in a bucket
@@ -1096,8 +1080,6 @@ OrderView order_view(uint64_t count, uint32_t wave, void* order) {
   v.sizes = w + kOrderHeadWords + L.nb1;
   v.ids = (const uint32_t*)((const char*)order + L.ids_off);
   v.nb = L.nb;
-  v.nb1 = L.nb1;
-  v.nb2 = L.nb2;
   v.room = L.room;
   return v;
 }
@@ -1309,7 +1291,6 @@ struct TileShared {
   uint32_t next;          // next place to take
 };
 constexpr uint32_t kDrawAgain = 0xFFFFFFFFu;  // instead of r - r0: r is drawn from the id
-
 
 template <int BS, bool Trace, bool Compact>
 __device__ __forceinline__ void sample_bucket(const SamplerArgs& A, const Plan& P, uint64_t W, uint32_t shift,
@@ -1580,13 +1561,12 @@ tc_status launch_sampler(const tc_graph* g, const Plan& plan, int64_t delta, con
   A.hash_mask = g->hash_mask;
   A.hash_shift = g->hash_shift;
   A.pair_t = g->pair_t;
-  A.pair_t32 = TC_COMPACT_PAIRS ? g->pair_t32 : nullptr;
+  A.pair_t32 = g->pair_t32;
   A.tmin = g->tmin;
   A.prefix = prefix;
   A.hdr = v.hdr;
   A.win = v.win;
   A.guide = v.guide;
-  A.k = k;
   A.chunk_base = 0;
   A.count = k;
   A.ord = OrderView{};
@@ -1669,7 +1649,7 @@ tc_status launch_path_sum(const tc_graph* g, const Plan& plan, int64_t delta, co
   A.hash_mask = g->hash_mask;
   A.hash_shift = g->hash_shift;
   A.pair_t = g->pair_t;
-  A.pair_t32 = TC_COMPACT_PAIRS ? g->pair_t32 : nullptr;
+  A.pair_t32 = g->pair_t32;
   A.tmin = g->tmin;
   A.prefix = prefix;
   A.hdr = v.hdr;
@@ -1724,13 +1704,12 @@ void batch_query_record(void* h_rec, const tc_graph* g, const Plan& plan, int64_
   A.hash_mask = g->hash_mask;
   A.hash_shift = g->hash_shift;
   A.pair_t = g->pair_t;
-  A.pair_t32 = TC_COMPACT_PAIRS ? g->pair_t32 : nullptr;
+  A.pair_t32 = g->pair_t32;
   A.tmin = g->tmin;
   A.prefix = prefix;
   A.hdr = v.hdr;
   A.win = v.win;
   A.guide = v.guide;
-  A.k = count;
   A.seed = seed;
   A.offset = offset;
   A.chunk_base = chunk_base;
