@@ -403,7 +403,9 @@ tc_status tc_mlp_train(tc_mlp* mlp, const tc_graph* g, const tc_motif* motif, in
  * TC_ERR_INVALID_ARG, as is an unknown objective); d_labels (grad) and the
  * sampled paths (train) carry the closure counts X.  For the variance
  * objective h_loss and h_losses receive the objective's value over the
- * rows or batch (not a per-row mean).  Device buffers are borrowed; the
+ * rows or batch (not a per-row mean).  Gradients and the variance objective
+ * are sums formed in no fixed order: their last bits may differ between two
+ * runs on the same inputs.  Device buffers are borrowed; the
  * calls allocate their scratch from the library's pool on the stream.
  */
 #define TC_OBJECTIVE_CLOSURE 0

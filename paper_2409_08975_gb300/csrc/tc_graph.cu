@@ -2,7 +2,7 @@
 // Sec. III-B: per-pair lists L_{u,v}) on the GPU, with this library's own
 // exclusive scans and stable LSD radix sort.
 //
-// Radix sort: least-significant-digit first, 8-bit digits, one pass =
+// Radix sort: least-significant-digit first, digits of up to 11 bits, one pass =
 // per-tile digit histograms, an exclusive scan of the digit-major histogram
 // table, and a stable scatter in which each warp ranks its keys with
 // __match_any_sync (warp-level multisplit) in input order.
@@ -462,8 +462,9 @@ tc_status radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v
 // the record's rank among the warp's earlier ones in the same sweep.
 //
 // Bound by the ranking's latency at 32 warps per SM (64 registers hold eight
-// records): 276 us per pass of 2e7 records (640 MB read and written, 94 us at
-// the copy rate) and 72 us for its histogram.  Passes over (key, index) pairs
+// records): 273 us per pass of 2e7 records on average (218 to 325 over the
+// nine passes; 640 MB read and written, 94 us at the copy rate) and 72 us for
+// its histogram (58 from the columns, 77 from records).  Passes over (key, index) pairs
 // took 227 + 58 us, but the gathers by the sorted permutations and the key
 // gathers before each sort another 2.7 ms in all.
 constexpr int kRecThreads = 512;
@@ -667,10 +668,12 @@ __device__ __forceinline__ void list_starts(uint32_t* off, int64_t prev, int64_t
 // The out-lists or the in-lists and the list starts from the sorted records.
 // Out: a record's id is its position in time order; the list's ids are the
 // input indexes found there, and canon[position in time order] receives the
-// canonical position for the in-lists' records.  Edges that follow one another
-// in a list lie close in time order, so this gather and scatter mostly stay
-// in a sector (30M edges of the transaction-like generator: 705 us, and 983 us
-// by input index with a further gather in the in-lists' first pass).
+// canonical position for the in-lists' records.  Bound by that gather and
+// scatter, a sector each for 4 bytes where neighbours in a list are far apart
+// in time order: 2e7 edges 628 us with 118 B read per edge, 3e8 edges 9.4 ms
+// with 137 B (the in-lists, which have neither, 124 us and 2.1 ms).  By input
+// index, with a further gather in the in-lists' first pass, they cost more
+// (30M edges of the transaction-like generator: 983 us, and 705 us this way).
 template <bool Out>
 __global__ void k_fill_list(const uint4* __restrict__ rec, const uint4* __restrict__ by_time, uint64_t m, int64_t n,
                             int64_t tmin, uint4* __restrict__ list, uint32_t* __restrict__ t32,

@@ -64,7 +64,9 @@ __host__ __device__ __forceinline__ uint64_t pair_key(uint32_t x, uint32_t y) {
 // First slot of the pair (x, y) in a pair table of 2^(64 - shift) slots (at
 // most 2^32: 2^31 distinct pairs alone exceed the device's memory): two
 // products, folded and multiplied once more, about ten instructions where the
-// 64-bit finaliser takes 25; the probe sequences are as short (mean 1.18 and
+// 64-bit finaliser takes 25 (multipliers: 2^64 over the golden ratio as in
+// Knuth's multiplicative hashing, the second prime of xxHash64, and that of
+// degski's 64-bit mixer); the probe sequences are as short (mean 1.18 and
 // 1.31 for present pairs of the two generators, 1.43 and 1.83 for absent ones,
 // both with either hash).
 __host__ __device__ __forceinline__ uint32_t pair_slot(uint32_t x, uint32_t y, int shift) {

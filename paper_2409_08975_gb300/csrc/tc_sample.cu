@@ -792,8 +792,8 @@ __device__ __forceinline__ void block_commit(SampleSums* G, uint64_t W, uint64_t
 // when a lane crosses into the next one (an edge has thousands of paths where
 // an exact count takes long), and the pair (p1, p3) is stepped on, so that a
 // path costs one coalesced end-edge load and its pair lookup.  Bound by issue
-// (62% of the slots, 97% of the loads hit L1); 4.0e9 paths of a 3e6-edge
-// graph: 26.2 ms (41.2 ms with a CDF search, a 64-bit division and both end
+// (67% of the slots at 1e6 edges, 97% of the loads hit L1); 4.0e9 paths of a
+// 3e6-edge graph: 24.8 ms, and in runs of a fixed 4096 26.2 ms (41.2 ms with a CDF search, a 64-bit division and both end
 // loads per path; 28.5 ms without pair_window's look at the list's ends).
 // Four blocks of 256 (64 registers): with five 29.9 ms, with six 33.9 ms.
 constexpr uint64_t kPathRun = 4096;  // a multiple of 32
